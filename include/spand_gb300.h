@@ -223,8 +223,8 @@ typedef struct {
    * programs                                                                */
   double t_host_phase_ms[8];
   /* the streaming RRQR kernel's memory traffic: bytes its column passes moved
-   * (each live column read and written once per pivot step; dead columns are
-   * skipped), in total and per level                                       */
+   * (an active column read and written once per pivot step, a column brought up
+   * to date once per bring-up), in total and per level                      */
   double rrqr_stream_bytes;
   double rrqr_stream_bytes_level[32];
 } spand_stats;

@@ -39,7 +39,7 @@
 
 namespace spand {
 
-// largest dynamic shared memory any kernel here asks for (x vectors, reflectors)
+// longest operand of one apply term (bytes): larger factors are refused
 constexpr size_t kGemvSmemMax = 200 * 1024;
 // dynamic shared memory of the RRQR cluster kernel (W chunk + reflector)
 constexpr size_t kQrSmemMax = 224 * 1024;   // clamped per kernel to the opt-in limit minus its static shared memory
@@ -599,40 +599,82 @@ static int qrs_capacity() {
   return coop ? std::min(nsm, QR_GMAX) : 0;
 }
 
-// register-resident rows of a column: 32 lanes x 16 bytes x NV
+// leading dimension of the reflectors: every column on 128-byte lines
 template <typename T>
-static int qrs_pick_nv(int nmax) {
-  constexpr int vw = 16 / sizeof(T);
-  for (int nv : {4, 8}) if (nmax <= 32 * vw * nv) return nv;
-  return 16;
+static int qrs_ldv(int n) {
+  constexpr int vw = 128 / sizeof(T);
+  return (n + vw - 1) / vw * vw;
 }
 
-// One cooperative launch of the streaming RRQR (one CTA per SM): the groups of
-// desc first, then a queue of single-CTA interfaces drained by every CTA.
-template <typename T, int NV>
-static int launch_stream_once(DevMem& tmp, const QrStreamTask<T>* dt, size_t nt, const std::vector<QrStreamTask<T>>& tasks,
-                              const std::vector<QrGroupDesc>& desc, const std::vector<int>& solo, int* d_flags, T eps,
-                              cudaStream_t st) {
-  auto kern = k_qrcp_stream<T, NV>;
-  int dev = 0, nsm = 0, per_sm = 0;
+// The streaming RRQR of a level's interfaces, in two launches that share the GPU:
+// groups of CTAs (a cooperative launch, one CTA per SM) for the interfaces with
+// more than a CTA's fair share of the work, and a queue of the others, one CTA
+// each, largest first, on the side stream.  A group gets as many CTAs as its
+// share of the work, but at most max(8, n / 16): an exchange costs 4 us at 8 to
+// 40 CTAs and 7 us at 57, and a step has about n / 4 active columns to deal out.
+// The queue has the SMs that are left and, as groups end, theirs.  Work is
+// estimated as n min(n, c) c (pivot steps x rows x columns), at the leaf level
+// times min(1, c / 30 n): there an interface with many large neighbours (a
+// junction of separators) keeps most of its rank, the others a tenth (256 x 128
+// p=3: ranks of 404 of 448 at c = 35 n, 32 to 60 of 448 at c = 10 n; above the
+// leaf level n has been through a compression and nearly all of it is kept).
+template <typename T>
+static int launch_qrcp_stream(DevMem& tmp, std::vector<QrStreamTask<T>>& tasks, int* d_flags, T eps,
+                              cudaStream_t st, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, bool leaf) {
+  int dev = 0, nsm = 0;
   SPAND_CUDA_TRY(cudaGetDevice(&dev));
   SPAND_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const int cap = std::min(nsm, QR_GMAX);
-  size_t smem = 0;
-  for (size_t d = 0; d < desc.size(); d += desc[d].G)
-    smem = std::max(smem, qrcp_stream_smem<T>(tasks[desc[d].task].ldw, tasks[desc[d].task].c, desc[d].G));
-  for (int i : solo) smem = std::max(smem, qrcp_stream_smem<T>(tasks[i].ldw, tasks[i].c, 1));
-  if (debug_level() >= 2) {
-    std::fprintf(stderr, "spand:   streaming launch: %zu group CTAs (", desc.size());
-    for (size_t d = 0; d < desc.size(); d += desc[d].G)
-      std::fprintf(stderr, " n%d c%d G%d", tasks[desc[d].task].n, tasks[desc[d].task].c, desc[d].G);
-    std::fprintf(stderr, " ), %zu single-CTA interfaces\n", solo.size());
+  const size_t nt = tasks.size();
+  std::vector<double> work(nt);
+  double wsum = 0;
+  for (size_t i = 0; i < nt; ++i) {
+    const double n = tasks[i].n, c = tasks[i].c;
+    work[i] = n * std::min(n, c) * c * (leaf ? std::min(1.0, c / (30.0 * n)) : 1.0);
+    wsum += work[i];
   }
-  if (set_dyn_smem((const void*)kern, smem) < (long long)smem) return SPAND_ERR_UNSUPPORTED;
-  SPAND_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, QRS_THREADS, smem));
-  if (per_sm < 1 || (int)desc.size() > cap) return SPAND_ERR_UNSUPPORTED;
-  QrGroupDesc* dd = desc.empty() ? nullptr : tmp.upload(desc);
-  int* ds = solo.empty() ? nullptr : tmp.upload(solo);
+  const double fair = wsum / cap;
+  std::vector<int> order(nt);
+  for (size_t i = 0; i < nt; ++i) order[i] = (int)i;
+  std::sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
+  std::vector<int> big, solo;
+  std::vector<QrGroupDesc> desc;
+  std::vector<int> gsize(nt, 1);
+  for (int i : order) {
+    const int G = std::min({(int)std::ceil(work[i] / fair), std::max(8, tasks[i].n / 16), tasks[i].c / 2,
+                            cap - (int)desc.size()});
+    if (G < 2) {
+      solo.push_back(i);
+      continue;
+    }
+    big.push_back(i);
+    gsize[i] = G;
+    for (int g = 0; g < G; ++g) desc.push_back({i, g, G, 0});
+  }
+  size_t ents = 0, grams = 0, smem_big = 0, smem_solo = 0;
+  auto lists = [&](size_t i) { return (size_t)gsize[i] * ((tasks[i].c + gsize[i] - 1) / gsize[i]); };
+  auto gram = [&](size_t i) { return (size_t)gsize[i] * std::min(tasks[i].n, tasks[i].c) * QRS_NB; };
+  for (size_t i = 0; i < nt; ++i) {
+    ents += lists(i);
+    grams += gram(i);
+  }
+  int* li = tmp.alloc<int>(ents * QRS_LISTS);
+  T* lv = tmp.alloc<T>(ents * QRS_VALS);
+  T* gr = tmp.alloc<T>(grams);
+  if (tmp.err) return SPAND_ERR_NOMEM;
+  ents = grams = 0;
+  for (size_t i = 0; i < nt; ++i) {
+    tasks[i].li = li + ents * QRS_LISTS;
+    tasks[i].lv = lv + ents * QRS_VALS;
+    tasks[i].gram = gr + grams;
+    ents += lists(i);
+    grams += gram(i);
+    size_t& sm = gsize[i] > 1 ? smem_big : smem_solo;
+    sm = std::max(sm, qrcp_stream_smem<T>(tasks[i].ldw, gsize[i] > 1));
+  }
+  const QrStreamTask<T>* dt = tmp.upload(tasks);
+  const QrGroupDesc* dd = desc.empty() ? nullptr : tmp.upload(desc);
+  const int* ds = solo.empty() ? nullptr : tmp.upload(solo);
   int* queue = tmp.alloc<int>(1);
   T* pv = tmp.alloc<T>(nt * 2 * QR_GMAX);
   int* pi = tmp.alloc<int>(nt * 2 * QR_GMAX);
@@ -641,89 +683,56 @@ static int launch_stream_once(DevMem& tmp, const QrStreamTask<T>* dt, size_t nt,
   if (tmp.err) return SPAND_ERR_NOMEM;
   SPAND_CUDA_TRY(cudaMemsetAsync(gs, 0, sizeof(GroupSync) * nt, st));
   SPAND_CUDA_TRY(cudaMemsetAsync(queue, 0, sizeof(int), st));
-  // every word starts with tag 255, which no word of steps 0 and 1 carries
+  // every word starts with tag 255, which no word of exchanges 0 and 1 carries
   SPAND_CUDA_TRY(cudaMemsetAsync(words, 0xFF, sizeof(unsigned long long) * nt * 2 * QR_GMAX, st));
   int poll_log2 = 22, fault_task = -1;
   if (take_barrier_fault()) {
     fault_task = desc.empty() ? solo[0] : desc[0].task;   // a partner that never arrives
     poll_log2 = 14;
   }
-  const int used = (int)desc.size();
-  const int grid = std::max(1, std::min(cap, used + (int)solo.size()));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(QRS_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  note_launch();
-  SPAND_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, dt, (const QrGroupDesc*)dd, used, (const int*)ds, (int)solo.size(),
-                                    queue, pv, pi, gs, words, d_flags, eps, poll_log2, fault_task));
-  return SPAND_OK;
-}
-
-template <typename T>
-static int launch_stream_nv(DevMem& tmp, const QrStreamTask<T>* dt, size_t nt, const std::vector<QrStreamTask<T>>& tasks,
-                            const std::vector<QrGroupDesc>& desc, const std::vector<int>& solo, int* d_flags, T eps,
-                            cudaStream_t st) {
-  int nmax = 0;
-  for (auto& d : desc) nmax = std::max(nmax, tasks[d.task].n);
-  for (int i : solo) nmax = std::max(nmax, tasks[i].n);
-  const int nv = qrs_pick_nv<T>(nmax);
-  if (nv <= 4) return launch_stream_once<T, 4>(tmp, dt, nt, tasks, desc, solo, d_flags, eps, st);
-  if (nv <= 8) return launch_stream_once<T, 8>(tmp, dt, nt, tasks, desc, solo, d_flags, eps, st);
-  return launch_stream_once<T, 16>(tmp, dt, nt, tasks, desc, solo, d_flags, eps, st);
-}
-
-// The streaming RRQR of a level's interfaces.  Interfaces with more than twice
-// a CTA's fair share of the work (estimated as n min(n, c) c: pivot steps x
-// rows x columns) are the critical path: they run first, in groups that
-// share every SM in proportion to their work; then every SM drains a queue of
-// the remaining interfaces one CTA each, largest first.
-template <typename T>
-static int launch_qrcp_stream(DevMem& tmp, const std::vector<QrStreamTask<T>>& tasks, int* d_flags, T eps,
-                              cudaStream_t st) {
-  int dev = 0, nsm = 0;
-  SPAND_CUDA_TRY(cudaGetDevice(&dev));
-  SPAND_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const int cap = std::min(nsm, QR_GMAX);
-  const size_t nt = tasks.size();
-  auto work = [&](int i) { return (double)tasks[i].n * std::min(tasks[i].n, tasks[i].c) * tasks[i].c; };
-  double wsum = 0;
-  for (size_t i = 0; i < nt; ++i) wsum += work((int)i);
-  const double fair = wsum / cap;
-  std::vector<int> order(nt);
-  for (size_t i = 0; i < nt; ++i) order[i] = (int)i;
-  std::sort(order.begin(), order.end(), [&](int a, int b) { return work(a) > work(b); });
-  std::vector<int> big, solo;
-  for (int i : order) {
-    if (work(i) > 2.0 * fair && tasks[i].c >= 2 && (int)big.size() < cap / 2) big.push_back(i);
-    else solo.push_back(i);
+  if (debug_level() >= 2) {
+    std::fprintf(stderr, "spand:   streaming launch: %zu group CTAs (", desc.size());
+    for (int b : big) std::fprintf(stderr, " n%d c%d G%d", tasks[b].n, tasks[b].c, gsize[b]);
+    std::fprintf(stderr, " ), %zu single-CTA interfaces\n", solo.size());
   }
-  QrStreamTask<T>* dt = tmp.upload(tasks);
-  if (tmp.err) return SPAND_ERR_NOMEM;
-  if (!big.empty()) {
-    // every SM over the large interfaces, in proportion to their work (>= 2 each)
-    double wb = 0;
-    for (int i : big) wb += work(i);
-    std::vector<int> G(big.size(), 2);
-    int left = cap - 2 * (int)big.size();
-    for (size_t b = 0; b < big.size(); ++b) {
-      const int extra = (int)std::floor((cap - 2.0 * big.size()) * work(big[b]) / wb);
-      const int add = std::max(0, std::min({extra, left, QR_GMAX - 2, tasks[big[b]].c - 2}));
-      G[b] += add;
-      left -= add;
-    }
-    std::vector<QrGroupDesc> desc;
-    for (size_t b = 0; b < big.size(); ++b)
-      for (int g = 0; g < G[b]; ++g) desc.push_back({big[b], g, G[b], 0});
-    SPAND_TRY(launch_stream_nv<T>(tmp, dt, nt, tasks, desc, std::vector<int>(), d_flags, eps, st));
+  const bool both = !desc.empty() && !solo.empty();
+  if (both) {
+    SPAND_CUDA_TRY(cudaEventRecord(fork, st));
+    SPAND_CUDA_TRY(cudaStreamWaitEvent(side, fork, 0));
   }
-  if (!solo.empty()) SPAND_TRY(launch_stream_nv<T>(tmp, dt, nt, tasks, std::vector<QrGroupDesc>(), solo, d_flags, eps, st));
+  if (!desc.empty()) {
+    auto kern = k_qrcp_stream_group<T>;
+    int per_sm = 0;
+    if (set_dyn_smem((const void*)kern, smem_big) < (long long)smem_big) return SPAND_ERR_UNSUPPORTED;
+    SPAND_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * qrs_warps(true), smem_big));
+    if (per_sm < 1 || (int)desc.size() > cap) return SPAND_ERR_UNSUPPORTED;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)desc.size(), 1, 1);
+    cfg.blockDim = dim3(32 * qrs_warps(true), 1, 1);
+    cfg.dynamicSmemBytes = smem_big;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    note_launch();
+    SPAND_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, dt, dd, pv, pi, gs, words, d_flags, eps, poll_log2, fault_task,
+                                      (int)smem_big));
+  }
+  if (!solo.empty()) {
+    auto kern = k_qrcp_stream_solo<T>;
+    if (set_dyn_smem((const void*)kern, smem_solo) < (long long)smem_solo) return SPAND_ERR_UNSUPPORTED;
+    const int grid = std::min(2 * cap, (int)solo.size());
+    note_launch();
+    kern<<<grid, 32 * qrs_warps(false), smem_solo, both ? side : st>>>(
+        dt, ds, (int)solo.size(), queue, pv, pi, gs, words, d_flags, eps, poll_log2, fault_task, (int)smem_solo);
+    SPAND_CUDA_TRY(cudaGetLastError());
+  }
+  if (both) {
+    SPAND_CUDA_TRY(cudaEventRecord(join, side));
+    SPAND_CUDA_TRY(cudaStreamWaitEvent(st, join, 0));
+  }
   return SPAND_OK;
 }
 
@@ -1640,7 +1649,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       if (nba[s].empty()) continue;
       int cs = 0;
       for (int b : nba[s]) cs += 2 * n[b];
-      vtot += (((size_t)n[s] * std::min(n[s], cs)) + 63) & ~size_t(63);
+      vtot += (((size_t)qrs_ldv<T>(n[s]) * std::min(n[s], cs)) + 63) & ~size_t(63);
     }
     T* vall = tmp.alloc<T>(std::max<size_t>(vtot, 1));
     if (tmp.err) return SPAND_ERR_NOMEM;
@@ -1658,7 +1667,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       // leading dimension padded to 16 bytes (the streaming kernel's form)
       t.W = tmp.alloc<T>((size_t)qrs_ldw<T>(n[s]) * cs);
       t.V = vall + voff;
-      voff += (((size_t)n[s] * std::min(n[s], cs)) + 63) & ~size_t(63);
+      voff += (((size_t)qrs_ldv<T>(n[s]) * std::min(n[s], cs)) + 63) & ~size_t(63);
       t.tau = tmp.alloc<T>(std::min(n[s], cs));
       t.norm2 = tmp.alloc<T>(cs);
       t.Q = nullptr;
@@ -1681,7 +1690,8 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       if (cs >= n[s]) flops += 2.0 * cs * (double)n[s] * n[s] - 2.0 / 3.0 * pow((double)n[s], 3);
     }
     if (tmp.err) return SPAND_ERR_NOMEM;
-    std::vector<int> rank(qt.size());
+    std::vector<int> rank(qt.size()), ldv(qt.size());    // ldv: leading dimension of each V
+    for (size_t q = 0; q < qt.size(); ++q) ldv[q] = qt[q].n;
     std::vector<std::array<int, 3>> strm_dbg;     // (n, c, index in qt) of the streamed interfaces (debug)
     std::vector<unsigned long long> strm_work;   // elements each streamed interface's passes moved
     int qf[4] = {0, 0, 0, 0};
@@ -1974,10 +1984,10 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
           u.W = t.W;
           u.V = t.V;
           u.tau = t.tau;
-          u.Q = nullptr;
           u.n = t.n;
           u.c = t.c;
           u.ldw = ldw;
+          u.ldv = ldv[qi] = qrs_ldv<T>(t.n);
           u.rank = t.rank;
           u.work = d_work + strm.size();
           strm.push_back(u);
@@ -2036,7 +2046,8 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
                                               d_flags, d_slots, slot_ns, (T)eps));
         }
       }
-      if (!strm.empty()) SPAND_TRY(launch_qrcp_stream<T>(tmp, strm, d_flags, (T)eps, st));
+      if (!strm.empty())
+        SPAND_TRY(launch_qrcp_stream<T>(tmp, strm, d_flags, (T)eps, st, sides.s[0], sides.fork, sides.join[0], l == 0));
       ev_end(ev_qr[l]);
       S.rrqr_launches += 1;
       SPAND_CUDA_TRY(cudaMemcpyAsync(rank.data(), d_rank, sizeof(int) * qt.size(), cudaMemcpyDeviceToHost, st));
@@ -2139,7 +2150,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
         T* G = tmp.alloc<T>((size_t)r * r);
         T* Tm = tmp.alloc<T>((size_t)r * r);
         T* M = tmp.alloc<T>((size_t)r * r);
-        gm.push_back({qt[q].V, qt[q].V, nn, nn, nn, 1, 0, 0});
+        gm.push_back({qt[q].V, qt[q].V, ldv[q], ldv[q], nn, 1, 0, 0});
         gt.push_back({G, r, r, r, (T)1, (T)0, (int)gm.size() - 1, (int)gm.size()});
         wy.push_back({G, qt[q].tau, r});
         MatRef<T> mr;
@@ -2150,10 +2161,10 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
         tri.push_back(mr);
         Tinv.push_back(Tm);
         nod.push_back(nullptr);
-        mm.push_back({Tm, qt[q].V, r, nn, r, 0, 1, 0});
+        mm.push_back({Tm, qt[q].V, r, ldv[q], r, 0, 1, 0});
         mt.push_back({M, r, r, r, (T)1, (T)0, (int)mm.size() - 1, (int)mm.size()});
         eye_q.push_back({qt[q].Q, nn, r, nn});     // Q_c = [I_r; 0] before the update below
-        qm.push_back({qt[q].V, M, nn, r, r, 0, 0, 0});
+        qm.push_back({qt[q].V, M, ldv[q], r, r, 0, 0, 0});
         qtk.push_back({qt[q].Q, nn, nn, r, (T)-1, (T)1, (int)qm.size() - 1, (int)qm.size()});
       }
       if (tmp.err) return SPAND_ERR_NOMEM;
