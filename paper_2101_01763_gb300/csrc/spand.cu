@@ -31,6 +31,7 @@
 
 #include "dense.cuh"
 #include "qrcp_stream.cuh"
+#include "gemm_split.cuh"
 #include "gemv.cuh"
 #include "umma.cuh"
 #include "umma2.cuh"
@@ -476,7 +477,17 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
     }
     if (e1) cudaEventRecord(e1, st);
   } else {
-    k_gemm<T><<<(unsigned)tiles.size(), 256, 0, st>>>(dt, dm, dl);
+    // the split kernel works in 64-wide chunks of k: below 48 values of k per
+    // product on average (the 32-wide LU updates) its chunks are mostly padding
+    double ks = 0;
+    for (const auto& tm : terms) ks += tm.k;
+    if (ks >= 48.0 * terms.size()) {
+      static std::atomic<uint64_t> attr64{0};
+      once_per_device(attr64, [] { set_dyn_smem((const void*)k_gemm_split, GS_SMEM_BYTES); });
+      k_gemm_split<<<(unsigned)tiles.size(), 256, GS_SMEM_BYTES, st>>>(dt, dm, dl);
+    } else {
+      k_gemm<T><<<(unsigned)tiles.size(), 256, 0, st>>>(dt, dm, dl);
+    }
   }
 }
 
