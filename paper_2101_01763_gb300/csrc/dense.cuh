@@ -239,54 +239,72 @@ __global__ void __launch_bounds__(256) k_getrf_panel(const MatRef<T>* mats, int 
 // The panel's interchanges as one row gather for the columns outside it:
 // after the swaps, row pos[i] holds what row src[i] held (rows relative to k0;
 // at most 2 jb rows move).  rec[0] = count, rec[1..] = pos, rec[1 + 2 LU_NB..]
-// = src.  One thread.
+// = src.  One warp: lane l holds the panel's own row l and the l-th other row
+// that moves, so an interchange is a ballot and two shuffles.  (One thread with
+// the lists in local memory took longer than the panel's 32 columns: 60 of 93 us
+// per panel at 64 x 32 p=2.)
 __device__ inline void lu_record_interchanges(int* rec, const int* piv_loc, int jb) {
-  int pos[2 * LU_NB], src[2 * LU_NB];
-  int cnt = 0;
-  for (int j = 0; j < jb; ++j) {
-    pos[cnt] = j;
-    src[cnt] = j;
-    ++cnt;
-  }
+  const int lane = threadIdx.x & 31;
+  int src0 = lane, pos1 = -1, src1 = -1, ne = 0;
   for (int j = 0; j < jb; ++j) {
     const int pj = piv_loc[j];
     if (pj == j) continue;
-    int a = -1, b = -1;
-    for (int t = 0; t < cnt; ++t) {
-      if (pos[t] == j) a = t;
-      if (pos[t] == pj) b = t;
+    const int sj = __shfl_sync(0xffffffffu, src0, j);
+    if (pj < jb) {
+      const int sp = __shfl_sync(0xffffffffu, src0, pj);
+      if (lane == j) src0 = sp;
+      if (lane == pj) src0 = sj;
+    } else {
+      const unsigned m = __ballot_sync(0xffffffffu, pos1 == pj);
+      const int t = m ? __ffs(m) - 1 : ne;
+      if (!m) {                      // first time row pj moves
+        if (lane == t) pos1 = src1 = pj;
+        ++ne;
+      }
+      const int sp = __shfl_sync(0xffffffffu, src1, t);
+      if (lane == j) src0 = sp;
+      if (lane == t) src1 = sj;
     }
-    if (b < 0) {                     // first time row pj moves
-      pos[cnt] = pj;
-      src[cnt] = pj;
-      b = cnt++;
-    }
-    const int t = src[a];
-    src[a] = src[b];
-    src[b] = t;
   }
-  rec[0] = cnt;
-  for (int t = 0; t < cnt; ++t) {
-    rec[1 + t] = pos[t];
-    rec[1 + 2 * LU_NB + t] = src[t];
+  if (lane == 0) rec[0] = jb + ne;
+  if (lane < jb) {
+    rec[1 + lane] = lane;
+    rec[1 + 2 * LU_NB + lane] = src0;
+  }
+  if (lane < ne) {
+    rec[1 + jb + lane] = pos1;
+    rec[1 + 2 * LU_NB + jb + lane] = src1;
   }
 }
 
 // The panel step of k_getrf_panel with the panel (rows k0..n-1 of the 32 panel
-// columns) staged in shared memory: pivot search, interchanges, scaling and the
-// rank-1 updates run on-chip; afterwards the panel is written back and the rows
-// its interchanges move are recorded for k_getrf_swap_trsm, which updates the
-// columns outside the panel.  Used when (n - k0) * 32 values fit the shared
+// columns) staged in shared memory; afterwards the panel is written back and the
+// rows its interchanges move are recorded for k_getrf_swap_trsm, which updates
+// the columns outside the panel.  Used when (n - k0) * 32 values fit the shared
 // budget.
+//
+// Bound: the latency of 32 dependent columns.  LU_SB columns at a time live in
+// registers (a thread owns rows tid, tid + 512, ...), so a column costs a pivot
+// reduction, one exchange of two rows through shared memory and multiply-adds;
+// the columns right of them take one rank-LU_SB update per block.  (With the
+// rank-1 updates in shared memory every column read and wrote the rest of the
+// panel: 8 MB at 2,048 rows against 1.3 MB.)  Each entry sees the same
+// operations in the same order as with rank-1 updates.
 constexpr int LU_SMEM_BYTES = 200 * 1024;
+constexpr int LU_SB = 8;
+constexpr int LU_PT = 512;                       // threads of the shared-memory panel
 
 template <typename T>
-__global__ void __launch_bounds__(512) k_getrf_panel_smem(const MatRef<T>* mats, int nmat, int k0, int* flags) {
+__global__ void __launch_bounds__(LU_PT) k_getrf_panel_smem(const MatRef<T>* mats, int nmat, int k0, int* flags) {
+  // rows per thread: the shared budget holds this many rows of 32 values
+  constexpr int RPT = (LU_SMEM_BYTES / (LU_NB * (int)sizeof(T)) + LU_PT - 1) / LU_PT;
   extern __shared__ unsigned char lu_smem[];
   T* P = reinterpret_cast<T*>(lu_smem);          // panel, column-major m x jb (ld m)
-  __shared__ T sv[32];
-  __shared__ int si[32];
+  __shared__ T sv[LU_PT / 32];
+  __shared__ int si[LU_PT / 32];
   __shared__ int piv_loc[LU_NB];
+  __shared__ T rowj[LU_SB], rowp[LU_SB];         // rows j and p of the block's columns
+  __shared__ T ub[LU_NB][LU_SB];                 // U of the block's rows in the columns right of it
   const int b = blockIdx.x;
   if (b >= nmat) return;
   const MatRef<T> M = mats[b];
@@ -295,78 +313,140 @@ __global__ void __launch_bounds__(512) k_getrf_panel_smem(const MatRef<T>* mats,
   T* A = M.A;
   const size_t ld = n;
   const int jb = min(LU_NB, n - k0), m = n - k0;
-  if ((size_t)m * jb * sizeof(T) > (size_t)LU_SMEM_BYTES) return;   // host routes these elsewhere
-  for (int idx = threadIdx.x; idx < m * jb; idx += blockDim.x) {
-    const int r = idx % m, c = idx / m;
-    P[idx] = A[(k0 + r) + (size_t)(k0 + c) * ld];
-  }
+  if ((size_t)m * jb * sizeof(T) > (size_t)LU_SMEM_BYTES || m > RPT * LU_PT) return;   // host routes these elsewhere
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int c = wid; c < jb; c += LU_PT / 32)
+    for (int r = lane; r < m; r += 32) P[r + c * m] = A[(k0 + r) + (size_t)(k0 + c) * ld];
   __syncthreads();
-  // pivot of column 0; later columns get theirs from the rank-1 update pass
-  // (each thread tracks |P(i, j+1)| of its rows as it updates them)
-  int p;
-  {
-    T best = -1;
-    int bi = m;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      T a = fabs(P[i]);
-      if (a != a) a = (T)INFINITY;
-      argmax_pair(best, bi, a, i);
+  for (int s0 = 0; s0 < jb; s0 += LU_SB) {
+    const int sb = min(LU_SB, jb - s0);
+    T x[RPT][LU_SB];
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+      const int i = tid + LU_PT * r;
+#pragma unroll
+      for (int c = 0; c < LU_SB; ++c) x[r][c] = (i < m && c < sb) ? P[i + (s0 + c) * m] : (T)0;
     }
-    block_argmax(best, bi, sv, si);
-    p = bi;
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int j = 0; j < jb; ++j) {
-    if (threadIdx.x == 0) {
-      M.ipiv[k0 + j] = k0 + p;
-      piv_loc[j] = p;
+#pragma unroll
+    for (int c = 0; c < LU_SB; ++c) {
+      if (c >= sb) break;
+      const int j = s0 + c;
+      // ---- pivot of column j (NaN ranks first so it is caught)
+      T best = -1;
+      int bi = m;
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        const int i = tid + LU_PT * r;
+        if (i >= j && i < m) {
+          T a = fabs(x[r][c]);
+          if (a != a) a = (T)INFINITY;
+          argmax_pair(best, bi, a, i);
+        }
+      }
+      warp_argmax(best, bi);
+      if (lane == 0) {
+        sv[wid] = best;
+        si[wid] = bi;
+      }
+      __syncthreads();
+      best = sv[lane & (LU_PT / 32 - 1)];
+      bi = si[lane & (LU_PT / 32 - 1)];
+      warp_argmax(best, bi);
+      const int p = bi;
+      if (tid == 0) {
+        M.ipiv[k0 + j] = k0 + p;
+        piv_loc[j] = p;
+      }
+      // ---- interchange rows j and p: the block's columns through rowj / rowp,
+      // the panel's other columns in place
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        const int i = tid + LU_PT * r;
+        if (i == j)
+#pragma unroll
+          for (int q = 0; q < LU_SB; ++q) rowj[q] = x[r][q];
+        if (i == p)
+#pragma unroll
+          for (int q = 0; q < LU_SB; ++q) rowp[q] = x[r][q];
+      }
+      if (p != j && wid == LU_PT / 32 - 1 && lane < jb && (lane < s0 || lane >= s0 + sb)) {
+        const T t = P[j + lane * m];
+        P[j + lane * m] = P[p + lane * m];
+        P[p + lane * m] = t;
+      }
+      __syncthreads();
+      T u[LU_SB];
+#pragma unroll
+      for (int q = 0; q < LU_SB; ++q) u[q] = rowp[q];
+      const T pv = u[c];
+      const bool bad = !(pv == pv) || isinf(pv) || pv == (T)0;
+      if (tid == 0 && bad) atomicOr(flags, (pv == (T)0) ? 1 : 2);
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        const int i = tid + LU_PT * r;
+        if (p != j && i == p)
+#pragma unroll
+          for (int q = 0; q < LU_SB; ++q) x[r][q] = rowj[q];
+        if (i == j) {
+#pragma unroll
+          for (int q = 0; q < LU_SB; ++q) x[r][q] = u[q];
+        } else if (i > j && i < m && !bad) {
+          const T l = x[r][c] / pv;
+          x[r][c] = l;
+#pragma unroll
+          for (int q = c + 1; q < LU_SB; ++q) x[r][q] -= l * u[q];
+        }
+      }
     }
-    if (p != j && threadIdx.x < jb) {
-      const int c = threadIdx.x;
-      const T t = P[j + c * m];
-      P[j + c * m] = P[p + c * m];
-      P[p + c * m] = t;
+    // ---- the block back to the panel
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+      const int i = tid + LU_PT * r;
+#pragma unroll
+      for (int c = 0; c < LU_SB; ++c)
+        if (i < m && c < sb) P[i + (s0 + c) * m] = x[r][c];
     }
     __syncthreads();
-    const T pv = P[j + j * m];
-    const bool bad = !(pv == pv) || isinf(pv) || pv == (T)0;
-    if (threadIdx.x == 0 && bad) atomicOr(flags, (pv == (T)0) ? 1 : 2);
-    T best = -1;
-    int bi = m;
-    for (int i = j + 1 + threadIdx.x; i < m; i += blockDim.x) {
-      if (!bad) {
-        const T l = P[i + j * m] / pv;
-        P[i + j * m] = l;
-        for (int c = j + 1; c < jb; ++c) P[i + c * m] -= l * P[j + c * m];
+    const int nc = jb - s0 - sb;                 // columns right of the block
+    if (nc <= 0) break;
+    // U of the block's rows (unit lower solve), a lane per column
+    if (wid == 0 && lane < nc) {
+      T* col = P + s0 + (s0 + sb + lane) * m;
+      T y[LU_SB];
+#pragma unroll
+      for (int q = 0; q < LU_SB; ++q) y[q] = q < sb ? col[q] : (T)0;
+#pragma unroll
+      for (int q = 0; q < LU_SB; ++q) {
+        const T pvq = q < sb ? P[(s0 + q) + (s0 + q) * m] : (T)0;
+        // a column whose pivot was zero or not finite updated nothing
+        const bool bad = !(pvq == pvq) || isinf(pvq) || pvq == (T)0;
+#pragma unroll
+        for (int t = q + 1; t < LU_SB; ++t)
+          if (t < sb && !bad) y[t] -= P[(s0 + t) + (s0 + q) * m] * y[q];
+        ub[lane][q] = bad ? (T)0 : y[q];
+        if (q < sb) col[q] = y[q];
       }
-      if (j + 1 < jb) {
-        T a = fabs(P[i + (j + 1) * m]);
-        if (a != a) a = (T)INFINITY;
-        argmax_pair(best, bi, a, i);
-      }
-    }
-    warp_argmax(best, bi);
-    if (lane == 0) {
-      sv[wid] = best;
-      si[wid] = bi;
     }
     __syncthreads();
-    // every thread combines the warps' candidates (read before the next
-    // iteration's first barrier, written only after it)
-    T b2 = -1;
-    int i2 = m;
-    for (int w = 0; w < nw; ++w) argmax_pair(b2, i2, sv[w], si[w]);
-    p = i2;
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+      const int i = tid + LU_PT * r;
+      if (i < s0 + sb || i >= m) continue;
+      for (int c = 0; c < nc; ++c) {
+        T a = P[i + (s0 + sb + c) * m];
+#pragma unroll
+        for (int q = 0; q < LU_SB; ++q) a -= x[r][q] * ub[c][q];
+        P[i + (s0 + sb + c) * m] = a;
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < m * jb; idx += blockDim.x) {
-    const int r = idx % m, c = idx / m;
-    A[(k0 + r) + (size_t)(k0 + c) * ld] = P[idx];
-  }
+  for (int c = wid; c < jb; c += LU_PT / 32)
+    for (int r = lane; r < m; r += 32) A[(k0 + r) + (size_t)(k0 + c) * ld] = P[r + c * m];
   // the panel's interchanges as one row gather for the columns outside it:
   // after the swaps, row pos[i] holds what row src[i] held (rows relative to
   // k0; at most 2 jb rows move).  Applied by k_getrf_swap_trsm.
-  if (threadIdx.x == 0) lu_record_interchanges(M.aff + (size_t)b * (1 + 4 * LU_NB), piv_loc, jb);
+  if (tid == 0) lu_record_interchanges(M.aff + (size_t)b * (1 + 4 * LU_NB), piv_loc, jb);
 }
 
 // The panel step with the panel's rows spread over the CTAs of a thread-block
@@ -492,7 +572,7 @@ __global__ void __launch_bounds__(512) k_getrf_panel_cl(const MatRef<T>* mats, i
     const int r = idx % nr, c = idx / nr;
     A[(k0 + r0 + r) + (size_t)(k0 + c) * ld] = P[r + c * R];
   }
-  if (rank == 0 && tid == 0) lu_record_interchanges(M.aff + (size_t)b * (1 + 4 * LU_NB), piv_loc, jb);
+  if (rank == 0 && tid < 32) lu_record_interchanges(M.aff + (size_t)b * (1 + 4 * LU_NB), piv_loc, jb);
   cl.sync();                                    // no CTA leaves while a peer may still address it
 }
 

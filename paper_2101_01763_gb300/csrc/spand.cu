@@ -852,7 +852,7 @@ static void batched_getrf(DevMem& tmp, std::vector<MatRef<T>>& mats, int* d_flag
     if (ds) {
       const size_t sm = (size_t)(nsmall_max - k0) * std::min(LU_NB, nsmall_max - k0) * sizeof(T);
       note_launch();
-      k_getrf_panel_smem<T><<<(unsigned)small.size(), 512, sm, st>>>(ds, (int)small.size(), k0, d_flags);
+      k_getrf_panel_smem<T><<<(unsigned)small.size(), LU_PT, sm, st>>>(ds, (int)small.size(), k0, d_flags);
       swap_trsm(small, ds, k0, tcol);
     }
     for (int q = 0; q < 3; ++q) {
