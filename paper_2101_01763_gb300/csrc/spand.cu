@@ -41,7 +41,7 @@
 namespace spand {
 
 // longest operand of one apply term (bytes): larger factors are refused
-constexpr size_t kGemvSmemMax = 200 * 1024;
+constexpr size_t kGemvTermMax = 200 * 1024;
 // dynamic shared memory of the RRQR cluster kernel (W chunk + reflector)
 constexpr size_t kQrSmemMax = 224 * 1024;   // clamped per kernel to the opt-in limit minus its static shared memory
 
@@ -1072,6 +1072,8 @@ struct ApplyProg {
     GvTile* tiles = nullptr;
     int ntiles = 0;
     int kmax = 0;
+    bool trans = false;        // matrices applied transposed
+    int groups = 1;            // 32-row groups per tile
   };
   std::vector<Phase> fwd, bwd;     // M^-1
   std::vector<Phase> tfwd, tbwd;   // M^-T
@@ -1085,6 +1087,8 @@ struct Program {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   int off = 0, N = 0;
   int64_t bytes = 0;          // factor bytes one apply reads
+  T* partial = nullptr;       // sums of the pieces of long tiles, their counters
+  int* done = nullptr;
   ~Program() {
     for (int t = 0; t < 2; ++t)
       if (graph[t]) cudaGraphExecDestroy(graph[t]);
@@ -2356,13 +2360,47 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
     }
   }
   typedef typename ApplyProg<T>::Phase Phase;
+  int gv_slots = 0;                        // partial sums the program's longest phase keeps
   auto build = [&](std::vector<GvTask<T>>& tasks, std::vector<GvTerm<T>>& terms) -> Phase {
     Phase ph;
     std::vector<GvTile> tiles;
+    for (auto& tm : terms) {
+      ph.kmax = std::max(ph.kmax, tm.k);
+      if (tm.M && tm.trans) ph.trans = true;
+    }
+    size_t n32 = 0;
+    for (auto& tk : tasks) n32 += (tk.m + GV_ROWS - 1) / GV_ROWS;
+    if (!ph.trans && n32 >= GV_MANY) ph.groups = 2;
+    // chunks of every tile; tiles much longer than the phase's even share are cut
+    int64_t all = 0;
+    int jlo, jhi;
     for (int t = 0; t < (int)tasks.size(); ++t)
-      for (int r0 = 0; r0 < tasks[t].m; r0 += GV_ROWS) tiles.push_back({t, r0});
-    for (auto& tm : terms) ph.kmax = std::max(ph.kmax, tm.k);
+      for (int r0 = 0; r0 < tasks[t].m; r0 += GV_ROWS * ph.groups) {
+        int n = 0;
+        for (int q = tasks[t].t0; q < tasks[t].t1; ++q)
+          n += ph.groups == 2 ? gv_chunks<2>(terms[q], r0, jlo, jhi) : gv_chunks<1>(terms[q], r0, jlo, jhi);
+        tiles.push_back({t, r0, 0, n, 0, 0, 1});
+        all += n;
+      }
     if (tiles.empty()) return ph;
+    const int piece = std::max<int>(GV_PIECE, (int)(all / GV_MANY));
+    const size_t whole = tiles.size();
+    int slots = 0;
+    for (size_t i = 0; i < whole; ++i) {
+      const GvTile tl = tiles[i];
+      const int ns = (tl.c1 + piece - 1) / piece;
+      if (ns < 2) continue;
+      for (int g = 0; g < ns; ++g) {
+        const GvTile cut{tl.task, tl.r0, (int)((int64_t)tl.c1 * g / ns), (int)((int64_t)tl.c1 * (g + 1) / ns), slots, g, ns};
+        if (g == 0) tiles[i] = cut;
+        else tiles.push_back(cut);
+      }
+      slots += ns;
+    }
+    gv_slots = std::max(gv_slots, slots);
+    // the longest pieces start first
+    std::stable_sort(tiles.begin(), tiles.end(),
+                     [](const GvTile& a, const GvTile& b) { return a.c1 - a.c0 > b.c1 - b.c0; });
     upload3(pm, tasks, terms, tiles, ph.tasks, ph.terms, ph.tiles);
     ph.ntiles = (int)tiles.size();
     return ph;
@@ -2373,6 +2411,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
   // sweeps of the clusters keep(l, c) selects (one system, or all of them)
   auto build_prog = [&](Program<T>& pg, auto keep) {
   int64_t& apply_bytes = pg.bytes;
+  gv_slots = 0;
   for (int tr = 0; tr < 2; ++tr) {
     std::vector<Phase>& fwd = tr ? pg.prog.tfwd : pg.prog.fwd;
     std::vector<Phase>& bwd = tr ? pg.prog.tbwd : pg.prog.bwd;
@@ -2553,6 +2592,11 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       }
     }
   }
+  if (gv_slots) {
+    pg.partial = pm.alloc<T>((size_t)gv_slots * 2 * GV_ROWS);
+    pg.done = pm.alloc<int>(gv_slots);
+    if (!pm.err && cudaMemsetAsync(pg.done, 0, sizeof(int) * gv_slots, st) != cudaSuccess) pm.err = 1;
+  }
   };
   F->progs.clear();
   {
@@ -2589,20 +2633,14 @@ __global__ void k_convert(const Tin* a, Tout* b, int n) {
 }
 
 template <typename T>
-static void gemv_attr() {
-  static std::atomic<uint64_t> attr{0};
-  once_per_device(attr, [] {
-    set_dyn_smem((const void*)k_gemv<T>, kGemvSmemMax);
-  });
-}
-
-template <typename T>
-static int run_phases(const std::vector<typename ApplyProg<T>::Phase>& ph, cudaStream_t st, bool capturing = false) {
-  gemv_attr<T>();
+static int run_phases(const Program<T>& pg, const std::vector<typename ApplyProg<T>::Phase>& ph, cudaStream_t st,
+                      bool capturing = false) {
   if (!capturing) note_launch(ph.size());
   for (auto& p : ph) {
-    const size_t sm = (size_t)std::max(p.kmax, 1) * sizeof(T);
-    k_gemv<T><<<p.ntiles, 256, sm, st>>>(p.tasks, p.terms, p.tiles);
+    // a phase of few tiles gets its parallelism from the warps of a tile
+    const int threads = p.ntiles < 600 ? 32 * GV_WARPS_MAX : 256;
+    auto kern = p.trans ? k_gemv<T, true, 1> : p.groups == 2 ? k_gemv<T, false, 2> : k_gemv<T, false, 1>;
+    kern<<<p.ntiles, threads, 0, st>>>(p.tasks, p.terms, p.tiles, pg.partial, pg.done);
   }
   return SPAND_OK;
 }
@@ -2626,19 +2664,18 @@ int apply_impl(FactorT<T>* F, Program<T>& pg, const double* r, double* zout, int
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   SPAND_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
   if (cs != cudaStreamCaptureStatusNone || direct) {
-    run_phases<T>(fwd, st);
-    run_phases<T>(bwd, st);
+    run_phases<T>(pg, fwd, st);
+    run_phases<T>(pg, bwd, st);
   } else {
     if (!pg.graph[d]) {
       // a private stream for the capture keeps the caller's stream untouched
       cudaStream_t cap;
       SPAND_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-      gemv_attr<T>();            // function attributes are not captured: set them first
       cudaGraph_t graph = nullptr;
       bool ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
       if (ok) {
-        run_phases<T>(fwd, cap, true);
-        run_phases<T>(bwd, cap, true);
+        run_phases<T>(pg, fwd, cap, true);
+        run_phases<T>(pg, bwd, cap, true);
         ok = cudaStreamEndCapture(cap, &graph) == cudaSuccess && graph;
       }
       if (ok) ok = cudaGraphInstantiate(&pg.graph[d], graph, 0) == cudaSuccess;
@@ -2651,8 +2688,8 @@ int apply_impl(FactorT<T>* F, Program<T>& pg, const double* r, double* zout, int
       note_launch(fwd.size() + bwd.size());
       SPAND_CUDA_TRY(cudaGraphLaunch(pg.graph[d], st));
     } else {
-      run_phases<T>(fwd, st);
-      run_phases<T>(bwd, st);
+      run_phases<T>(pg, fwd, st);
+      run_phases<T>(pg, bwd, st);
     }
   }
   if (zout) {                   // zout == nullptr: the caller reads the factor's vector itself
@@ -2680,12 +2717,12 @@ static int factor_any(const Plan& U, const bsr_matrix* const* As, double eps, in
     auto F = std::make_shared<FactorT<double>>();
     out = F;
     st = factor_impl<double>(U, As, eps, precision, F.get(), stream);
-    if (st == SPAND_OK && (size_t)max_kmax(F.get()) * sizeof(double) > kGemvSmemMax) st = SPAND_ERR_UNSUPPORTED;
+    if (st == SPAND_OK && (size_t)max_kmax(F.get()) * sizeof(double) > kGemvTermMax) st = SPAND_ERR_UNSUPPORTED;
   } else {
     auto F = std::make_shared<FactorT<float>>();
     out = F;
     st = factor_impl<float>(U, As, eps, precision, F.get(), stream);
-    if (st == SPAND_OK && (size_t)max_kmax(F.get()) * sizeof(float) > kGemvSmemMax) st = SPAND_ERR_UNSUPPORTED;
+    if (st == SPAND_OK && (size_t)max_kmax(F.get()) * sizeof(float) > kGemvTermMax) st = SPAND_ERR_UNSUPPORTED;
   }
   if (st != SPAND_OK) {
     cudaStreamSynchronize(stream);
