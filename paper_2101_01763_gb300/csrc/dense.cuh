@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(LU_PT) k_getrf_panel_smem(const MatRef<T>* mat
   // the panel's interchanges as one row gather for the columns outside it:
   // after the swaps, row pos[i] holds what row src[i] held (rows relative to
   // k0; at most 2 jb rows move).  Applied by k_getrf_swap_trsm.
-  if (tid == 0) lu_record_interchanges(M.aff + (size_t)b * (1 + 4 * LU_NB), piv_loc, jb);
+  if (tid < 32) lu_record_interchanges(M.aff + (size_t)b * (1 + 4 * LU_NB), piv_loc, jb);
 }
 
 // The panel step with the panel's rows spread over the CTAs of a thread-block
