@@ -20,6 +20,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <tuple>
 #include <mutex>
@@ -106,6 +107,7 @@ struct PinnedStage {
   static constexpr size_t kChunk = size_t(8) << 20;
   std::vector<std::pair<char*, size_t>> chunks;
   size_t ci = 0, off = 0;
+  unsigned gen = 0;                         // resets so far
   // host buffer for `bytes`, or nullptr (the caller then copies from pageable memory)
   char* get(size_t bytes) {
     bytes = (bytes + 63) & ~size_t(63);
@@ -138,6 +140,7 @@ struct PinnedStage {
   void reset() {   // only after the stream that read the chunks has been synchronised
     ci = 0;
     off = 0;
+    ++gen;
   }
   ~PinnedStage() {
     for (auto& c : chunks) PinnedPool::get().give(c);
@@ -147,6 +150,13 @@ struct PinnedStage {
 // Stream-ordered device memory carved from 32 MB slabs (256-byte aligned
 // pieces), so that the thousands of small arrays of a factorization cost a
 // handful of allocator calls; large arrays get their own allocation.
+//
+// Task tables of a chain of launches (the panels of an LU, the levels of the
+// inverses) are known before the chain starts.  Inside a Deferred scope, upload()
+// only writes them to a pinned buffer that mirrors a device buffer and run() only
+// notes the launch; one copy then carries the tables of many launches.  A copy
+// between two launches costs 6 us on the stream (copy + kernel 9.3 us, kernel
+// alone 3.0 us).
 struct DevMem {
   static constexpr size_t kSlab = size_t(32) << 20;
   std::vector<void*> ptrs;
@@ -155,6 +165,35 @@ struct DevMem {
   char* cur = nullptr;
   size_t left = 0;
   PinnedStage* stage = nullptr;   // optional pinned staging for uploads
+  static constexpr size_t kMirror = size_t(1) << 20;
+  int deferred = 0;               // open Deferred scopes
+  char *mh = nullptr, *md = nullptr;        // the mirrored buffers (host, device)
+  size_t m_used = 0, m_sent = 0;
+  unsigned m_gen = 0;
+  std::vector<std::function<void()>> queue;
+  // the tables written since the last call go to the device
+  void send() {
+    if (m_used > m_sent &&
+        cudaMemcpyAsync(md + m_sent, mh + m_sent, m_used - m_sent, cudaMemcpyHostToDevice, st) != cudaSuccess)
+      err = 1;
+    m_sent = m_used;
+  }
+  void go() {
+    send();
+    for (auto& f : queue)
+      if (!err) f();
+    queue.clear();
+  }
+  // launches f now, or with the scope's next batch
+  template <typename F>
+  void run(F f) {
+    if (!deferred) {
+      f();
+      return;
+    }
+    queue.emplace_back(std::move(f));
+    if (queue.size() >= 64) go();
+  }
   template <typename X>
   X* alloc(size_t n) {
     if (n == 0) n = 1;
@@ -186,9 +225,27 @@ struct DevMem {
   }
   template <typename X>
   X* upload(const std::vector<X>& h) {
+    const size_t bytes = h.size() * sizeof(X);
+    if (deferred && stage && bytes > 0 && bytes <= kMirror / 4) {
+      const size_t room = (bytes + 255) & ~size_t(255);
+      if (!mh || m_gen != stage->gen || m_used + room > kMirror) {
+        send();
+        mh = stage->get(kMirror);
+        md = mh ? alloc<char>(kMirror) : nullptr;
+        m_used = m_sent = 0;
+        m_gen = stage->gen;
+      }
+      if (md) {
+        memcpy(mh + m_used, h.data(), bytes);
+        X* d = reinterpret_cast<X*>(md + m_used);
+        m_used += room;
+        if (m_used - m_sent > kMirror / 4) go();     // a batch's tables: do not keep the GPU waiting for more
+        return d;
+      }
+      mh = nullptr;
+    }
     X* d = alloc<X>(h.size());
     if (!d || h.empty()) return d;
-    const size_t bytes = h.size() * sizeof(X);
     const void* src = h.data();
     if (stage) {
       char* p = stage->get(bytes);
@@ -205,6 +262,16 @@ struct DevMem {
     ptrs.clear();
     cur = nullptr;
     left = 0;
+    mh = md = nullptr;
+    m_used = m_sent = 0;
+  }
+};
+
+struct Deferred {
+  DevMem& m;
+  explicit Deferred(DevMem& mem) : m(mem) { ++m.deferred; }
+  ~Deferred() {
+    if (--m.deferred == 0) m.go();
   }
 };
 
@@ -290,6 +357,7 @@ struct GemmTuner {
   struct Entry {
     int choice = -1;                 // decided: 0 tcgen05, 1 mma.sync
     bool pending[2] = {false, false};
+    bool recorded[2] = {false, false};   // both events are on the stream
     bool done[2] = {false, false};
     double per_flop[2] = {0, 0};
     double flops[2] = {0, 0};
@@ -304,9 +372,10 @@ struct GemmTuner {
 };
 
 // returns the kernel (0 tcgen05, 1 mma.sync) and, when this launch is to be
-// timed, the two events to record around it
-static int gemm_pick(double avg_chunks, double flops, cudaEvent_t& e0, cudaEvent_t& e1) {
+// timed, the two events to record around it and the flag to set then
+static int gemm_pick(double avg_chunks, double flops, cudaEvent_t& e0, cudaEvent_t& e1, bool*& recorded) {
   e0 = e1 = nullptr;
+  recorded = nullptr;
   const int rule = avg_chunks >= 4.0 ? 0 : 1;
   if (gemm_mode() == 1) return 0;
   if (gemm_mode() == 2) return 1;
@@ -319,7 +388,7 @@ static int gemm_pick(double avg_chunks, double flops, cudaEvent_t& e0, cudaEvent
   GemmTuner::Entry& E = T.table[std::make_tuple(dev, cb, fb)];
   if (E.choice >= 0) return E.choice;
   for (int c = 0; c < 2; ++c)
-    if (E.pending[c] && !E.done[c]) {
+    if (E.pending[c] && E.recorded[c] && !E.done[c]) {
       const cudaError_t q = cudaEventQuery(E.ev[c][1]);
       if (q == cudaSuccess) {
         float ms = 0.f;
@@ -327,7 +396,7 @@ static int gemm_pick(double avg_chunks, double flops, cudaEvent_t& e0, cudaEvent
           E.per_flop[c] = ms / E.flops[c];
           E.done[c] = true;
         }
-        E.pending[c] = false;
+        E.pending[c] = E.recorded[c] = false;
       } else if (q == cudaErrorNotReady && cudaPeekAtLastError() == cudaErrorNotReady) {
         cudaGetLastError();          // a not-ready query is not an error of ours
       }
@@ -358,6 +427,7 @@ static int gemm_pick(double avg_chunks, double flops, cudaEvent_t& e0, cudaEvent
       E.flops[c] = flops;
       e0 = E.ev[c][0];
       e1 = E.ev[c][1];
+      recorded = &E.recorded[c];
       return c;
     }
   return rule;                       // both measurements still in flight
@@ -411,6 +481,7 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
                         cudaStream_t st, const char* tag = "") {
   bool umma = false;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
+  bool* recorded = nullptr;
   if (std::is_same<T, float>::value) {
     double chunks = 0, flops = 0;
     int ntask = 0;
@@ -422,7 +493,7 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
       }
       ++ntask;
     }
-    if (ntask > 0) umma = gemm_pick(chunks / ntask, flops, e0, e1) == 0;
+    if (ntask > 0) umma = gemm_pick(chunks / ntask, flops, e0, e1, recorded) == 0;
   }
   const int uv = umma_variant();
   const int BM = umma ? (uv == 2 ? U2_BM : UM_BM) : 64, BN = umma ? (uv == 2 ? U2_BN : UM_BN) : 64;
@@ -438,57 +509,64 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
   TileItem* dl;
   upload3(tmp, tasks, terms, tiles, dt, dm, dl);
   if (tmp.err) return;
-  note_launch();
   GemmLog::Rec rec{tag, std::is_same<T, float>::value ? (umma ? 0 : 1) : 2, 0.0, tiles.size(), nullptr, nullptr};
-  const bool logit = debug_level() >= 3 && cudaEventCreate(&rec.a) == cudaSuccess &&
-                     cudaEventCreate(&rec.b) == cudaSuccess && cudaEventRecord(rec.a, st) == cudaSuccess;
-  if (logit)
+  if (debug_level() >= 3)
     for (const auto& tk : tasks)
       for (int t = tk.t0; t < tk.t1; ++t)   // a triangular operand halves the useful flops
         rec.flops += (terms[t].tri ? 1.0 : 2.0) * tk.m * (double)tk.n * terms[t].k;
-  struct LogAtEnd {
-    bool on;
-    GemmLog::Rec& r;
-    cudaStream_t s;
-    ~LogAtEnd() {
-      if (on && cudaEventRecord(r.b, s) == cudaSuccess) GemmLog::get().recs.push_back(r);
-    }
-  } log_at_end{logit, rec, st};
-  if constexpr (std::is_same<T, float>::value) {
-    if (e0) cudaEventRecord(e0, st);
-    if (umma && uv == 1 && umma_depth() == 2) {
-      static std::atomic<uint64_t> attr{0};
-      once_per_device(attr, [] { set_dyn_smem((const void*)k_gemm_umma<2>, UM_SMEM_BYTES); });
-      k_gemm_umma<2><<<(unsigned)tiles.size(), 128, UM_SMEM_BYTES, st>>>(dt, dm, dl);
-    } else if (umma && uv == 1) {
-      static std::atomic<uint64_t> attr1{0};
-      once_per_device(attr1, [] { set_dyn_smem((const void*)k_gemm_umma<1>, UM_SMEM_BYTES); });
-      k_gemm_umma<1><<<(unsigned)tiles.size(), 128, UM_SMEM_BYTES, st>>>(dt, dm, dl);
-    } else if (umma && uv == 3) {
-      static std::atomic<uint64_t> attr3{0};
-      once_per_device(attr3, [] { set_dyn_smem((const void*)k_gemm_umma3, U3_SMEM_BYTES); });
-      k_gemm_umma3<<<(unsigned)tiles.size(), U3_THREADS, U3_SMEM_BYTES, st>>>(dt, dm, dl);
-    } else if (umma) {
-      static std::atomic<uint64_t> attr2{0};
-      once_per_device(attr2, [] { set_dyn_smem((const void*)k_gemm_umma2, U2_SMEM_BYTES); });
-      k_gemm_umma2<<<(unsigned)tiles.size(), 128, U2_SMEM_BYTES, st>>>(dt, dm, dl);
+  double ks = 0;
+  for (const auto& tm : terms) ks += tm.k;
+  const bool split = ks >= 48.0 * terms.size();
+  const unsigned ntiles = (unsigned)tiles.size();
+  tmp.run([=]() mutable {
+    note_launch();
+    const bool logit = debug_level() >= 3 && cudaEventCreate(&rec.a) == cudaSuccess &&
+                       cudaEventCreate(&rec.b) == cudaSuccess && cudaEventRecord(rec.a, st) == cudaSuccess;
+    struct LogAtEnd {
+      bool on;
+      GemmLog::Rec& r;
+      cudaStream_t s;
+      ~LogAtEnd() {
+        if (on && cudaEventRecord(r.b, s) == cudaSuccess) GemmLog::get().recs.push_back(r);
+      }
+    } log_at_end{logit, rec, st};
+    if constexpr (std::is_same<T, float>::value) {
+      if (e0) cudaEventRecord(e0, st);
+      if (umma && uv == 1 && umma_depth() == 2) {
+        static std::atomic<uint64_t> attr{0};
+        once_per_device(attr, [] { set_dyn_smem((const void*)k_gemm_umma<2>, UM_SMEM_BYTES); });
+        k_gemm_umma<2><<<ntiles, 128, UM_SMEM_BYTES, st>>>(dt, dm, dl);
+      } else if (umma && uv == 1) {
+        static std::atomic<uint64_t> attr1{0};
+        once_per_device(attr1, [] { set_dyn_smem((const void*)k_gemm_umma<1>, UM_SMEM_BYTES); });
+        k_gemm_umma<1><<<ntiles, 128, UM_SMEM_BYTES, st>>>(dt, dm, dl);
+      } else if (umma && uv == 3) {
+        static std::atomic<uint64_t> attr3{0};
+        once_per_device(attr3, [] { set_dyn_smem((const void*)k_gemm_umma3, U3_SMEM_BYTES); });
+        k_gemm_umma3<<<ntiles, U3_THREADS, U3_SMEM_BYTES, st>>>(dt, dm, dl);
+      } else if (umma) {
+        static std::atomic<uint64_t> attr2{0};
+        once_per_device(attr2, [] { set_dyn_smem((const void*)k_gemm_umma2, U2_SMEM_BYTES); });
+        k_gemm_umma2<<<ntiles, 128, U2_SMEM_BYTES, st>>>(dt, dm, dl);
+      } else {
+        k_gemm_tc<3><<<ntiles, 128, 0, st>>>(dt, dm, dl);   // 3xTF32 on mma.sync
+      }
+      if (e1 && cudaEventRecord(e1, st) == cudaSuccess) {
+        std::lock_guard<std::mutex> g(GemmTuner::get().mu);
+        *recorded = true;
+      }
     } else {
-      k_gemm_tc<3><<<(unsigned)tiles.size(), 128, 0, st>>>(dt, dm, dl);   // 3xTF32 on mma.sync
+      // the split kernel works in 64-wide chunks of k: below 48 values of k per
+      // product on average (the 32-wide LU updates) its chunks are mostly padding
+      if (split) {
+        static std::atomic<uint64_t> attr64{0};
+        once_per_device(attr64, [] { set_dyn_smem((const void*)k_gemm_split, GS_SMEM_BYTES); });
+        k_gemm_split<<<ntiles, 256, GS_SMEM_BYTES, st>>>(dt, dm, dl);
+      } else {
+        k_gemm<T><<<ntiles, 256, 0, st>>>(dt, dm, dl);
+      }
     }
-    if (e1) cudaEventRecord(e1, st);
-  } else {
-    // the split kernel works in 64-wide chunks of k: below 48 values of k per
-    // product on average (the 32-wide LU updates) its chunks are mostly padding
-    double ks = 0;
-    for (const auto& tm : terms) ks += tm.k;
-    if (ks >= 48.0 * terms.size()) {
-      static std::atomic<uint64_t> attr64{0};
-      once_per_device(attr64, [] { set_dyn_smem((const void*)k_gemm_split, GS_SMEM_BYTES); });
-      k_gemm_split<<<(unsigned)tiles.size(), 256, GS_SMEM_BYTES, st>>>(dt, dm, dl);
-    } else {
-      k_gemm<T><<<(unsigned)tiles.size(), 256, 0, st>>>(dt, dm, dl);
-    }
-  }
+  });
 }
 
 template <typename T>
@@ -502,8 +580,11 @@ static void launch_copy(DevMem& tmp, const std::vector<CopyTask<T>>& tasks, cuda
   CopyTile* dl;
   upload2(tmp, tasks, tiles, dt, dl);
   if (tmp.err) return;
-  note_launch();
-  k_copy_tiles<T><<<(unsigned)tiles.size(), 256, 0, st>>>(dt, dl);
+  const unsigned n = (unsigned)tiles.size();
+  tmp.run([=] {
+    note_launch();
+    k_copy_tiles<T><<<n, 256, 0, st>>>(dt, dl);
+  });
 }
 
 // row-permuted copy: dst[r, c] = src[perm[r], c]; one CTA per 64 x 32 tile
@@ -559,8 +640,11 @@ static void launch_row_perm(DevMem& tmp, const std::vector<const T*>& src, const
   RowPermTile* dl;
   upload2(tmp, tasks, tiles, dt, dl);
   if (tmp.err) return;
-  note_launch();
-  k_row_perm<T><<<(unsigned)tiles.size(), 256, 0, st>>>(dt, dl);
+  const unsigned n = (unsigned)tiles.size();
+  tmp.run([=] {
+    note_launch();
+    k_row_perm<T><<<n, 256, 0, st>>>(dt, dl);
+  });
 }
 
 // ------------------------------------------------------------------ streaming RRQR launch
@@ -766,6 +850,7 @@ constexpr int LU_CL_ROWS = 256;  // panel rows per cluster CTA aimed at
 template <typename T>
 static void batched_getrf(DevMem& tmp, std::vector<MatRef<T>>& mats, int* d_flags, cudaStream_t st) {
   if (mats.empty()) return;
+  Deferred chain(tmp);
   int nmax = 0;
   for (auto& m : mats) nmax = std::max(nmax, m.n);
   auto* dm = tmp.upload(mats);
@@ -796,8 +881,11 @@ static void batched_getrf(DevMem& tmp, std::vector<MatRef<T>>& mats, int* d_flag
     if (tl.empty()) return;
     auto* dtl = tmp.upload(tl);
     if (tmp.err) return;
-    note_launch();
-    k_getrf_swap_trsm<T><<<(unsigned)tl.size(), 256, 0, st>>>(dlist, dtl, k0, tcol);
+    const unsigned nt = (unsigned)tl.size();
+    tmp.run([=] {
+      note_launch();
+      k_getrf_swap_trsm<T><<<nt, 256, 0, st>>>(dlist, dtl, k0, tcol);
+    });
   };
   // Two-level blocking (the arrangement of LAPACK's blocked getrf): panels of
   // LU_NB columns are grouped in blocks of LU_NB2.  Inside a block a panel's
@@ -851,8 +939,11 @@ static void batched_getrf(DevMem& tmp, std::vector<MatRef<T>>& mats, int* d_flag
     if (tmp.err) return;
     if (ds) {
       const size_t sm = (size_t)(nsmall_max - k0) * std::min(LU_NB, nsmall_max - k0) * sizeof(T);
-      note_launch();
-      k_getrf_panel_smem<T><<<(unsigned)small.size(), LU_PT, sm, st>>>(ds, (int)small.size(), k0, d_flags);
+      const int nm = (int)small.size();
+      tmp.run([=] {
+        note_launch();
+        k_getrf_panel_smem<T><<<(unsigned)nm, LU_PT, sm, st>>>(ds, nm, k0, d_flags);
+      });
       swap_trsm(small, ds, k0, tcol);
     }
     for (int q = 0; q < 3; ++q) {
@@ -860,29 +951,34 @@ static void batched_getrf(DevMem& tmp, std::vector<MatRef<T>>& mats, int* d_flag
       const int C = 2 << q;
       auto* dc = tmp.upload(clus[q]);
       if (tmp.err) return;
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = C;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.gridDim = dim3((unsigned)(clus[q].size() * C), 1, 1);
-      cfg.blockDim = dim3(512, 1, 1);
-      cfg.dynamicSmemBytes = lu_cl_smem<T>((ncl_max[q] + C - 1) / C);
-      cfg.stream = st;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      note_launch();
-      if (cudaLaunchKernelEx(&cfg, k_getrf_panel_cl<T>, (const MatRef<T>*)dc, (int)clus[q].size(), k0, d_flags) !=
-          cudaSuccess) {
-        tmp.err = 1;
-        return;
-      }
+      const int nm = (int)clus[q].size();
+      const size_t sm = lu_cl_smem<T>((ncl_max[q] + C - 1) / C);
+      DevMem* mem = &tmp;
+      tmp.run([=] {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)(nm * C), 1, 1);
+        cfg.blockDim = dim3(512, 1, 1);
+        cfg.dynamicSmemBytes = sm;
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        note_launch();
+        if (cudaLaunchKernelEx(&cfg, k_getrf_panel_cl<T>, (const MatRef<T>*)dc, nm, k0, d_flags) != cudaSuccess)
+          mem->err = 1;
+      });
       swap_trsm(clus[q], dc, k0, tcol);
     }
     if (dlg) {
-      note_launch();
-      k_getrf_panel<T><<<(unsigned)large.size(), 256, 0, st>>>(dlg, (int)large.size(), k0, tcol, d_flags);
+      const int nm = (int)large.size();
+      tmp.run([=] {
+        note_launch();
+        k_getrf_panel<T><<<(unsigned)nm, 256, 0, st>>>(dlg, nm, k0, tcol, d_flags);
+      });
     }
     // rank-LU_NB update of the block's columns [r, Ke), every row below the panel
     std::vector<GemmTask<T>> tasks;
@@ -927,8 +1023,11 @@ static void batched_getrf(DevMem& tmp, std::vector<MatRef<T>>& mats, int* d_flag
       auto* dsub = tmp.upload(sub);
       auto* dtl = tmp.upload(tl);
       if (tmp.err) return;
-      note_launch();
-      k_lu_trsm_cols<T><<<(unsigned)tl.size(), 256, 0, st>>>(dsub, dtl, p0);
+      const unsigned nt = (unsigned)tl.size();
+      tmp.run([=] {
+        note_launch();
+        k_lu_trsm_cols<T><<<nt, 256, 0, st>>>(dsub, dtl, p0);
+      });
       launch_gemm(tmp, rt, rm, st, "lu-block-rows");
     }
     std::vector<GemmTask<T>> bt;
@@ -942,8 +1041,11 @@ static void batched_getrf(DevMem& tmp, std::vector<MatRef<T>>& mats, int* d_flag
     }
     launch_gemm(tmp, bt, bm, st, "lu-block");
   }
-  note_launch();
-  k_ipiv_to_perm<T><<<(unsigned)mats.size(), 128, (size_t)nmax * sizeof(int), st>>>(dm, (int)mats.size());
+  const int nm = (int)mats.size();
+  tmp.run([=] {
+    note_launch();
+    k_ipiv_to_perm<T><<<(unsigned)nm, 128, (size_t)nmax * sizeof(int), st>>>(dm, nm);
+  });
 }
 
 // L^-1 (optionally row-scaled by 1/d) and U^-1 (optionally column-scaled by d)
@@ -954,6 +1056,7 @@ template <typename T>
 static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, const std::vector<T*>& Linv,
                              const std::vector<T*>& Uinv, const std::vector<const T*>& dscale, cudaStream_t st) {
   if (mats.empty()) return;
+  Deferred chain(tmp);
   // zero both outputs (the opposite triangles must read as zeros)
   {
     std::vector<T*> ptr;
@@ -969,8 +1072,10 @@ static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, co
     if (tmp.err) return;
     for (size_t off = 0; off < ptr.size(); off += 65535) {
       const unsigned cnt = (unsigned)std::min<size_t>(65535, ptr.size() - off);
-      note_launch();
-      k_zero_mats<T><<<dim3(32, cnt), 256, 0, st>>>(dp + off, dn + off);
+      tmp.run([=] {
+        note_launch();
+        k_zero_mats<T><<<dim3(32, cnt), 256, 0, st>>>(dp + off, dn + off);
+      });
     }
   }
   std::vector<DiagInvTask<T>> dt;
@@ -986,8 +1091,11 @@ static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, co
   if (!dt.empty()) {
     auto* dd = tmp.upload(dt);
     if (tmp.err) return;
-    note_launch();
-    k_inv_diag<T><<<(unsigned)dt.size(), 32, 0, st>>>(dd);
+    const unsigned nd = (unsigned)dt.size();
+    tmp.run([=] {
+      note_launch();
+      k_inv_diag<T><<<nd, 32, 0, st>>>(dd);
+    });
   }
   for (int bs = 32; bs < nmax; bs *= 2) {
     // one scratch array per level for the products L21 X11 and U12 Y22
@@ -1039,10 +1147,13 @@ static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, co
   auto* dut = tmp.upload(ut);
   auto* dtl = tmp.upload(tiles);
   if (tmp.err) return;
-  note_launch();
-  k_scale_rows<T><<<(unsigned)tiles.size(), 256, 0, st>>>(dlt, dtl);
-  note_launch();
-  k_scale_cols<T><<<(unsigned)tiles.size(), 256, 0, st>>>(dut, dtl);
+  const unsigned nt = (unsigned)tiles.size();
+  tmp.run([=] {
+    note_launch();
+    k_scale_rows<T><<<nt, 256, 0, st>>>(dlt, dtl);
+    note_launch();
+    k_scale_cols<T><<<nt, 256, 0, st>>>(dut, dtl);
+  });
 }
 
 // U^-1 only (no permutation, no scaling)
@@ -1059,8 +1170,11 @@ static void batched_upper_inverse(DevMem& tmp, const std::vector<MatRef<T>>& mat
   auto* dut = tmp.upload(ut);
   auto* dtl = tmp.upload(tiles);
   if (tmp.err || tiles.empty()) return;
-  note_launch();
-  k_inv_upper<T><<<(unsigned)tiles.size(), 256, 0, st>>>(dut, dtl);
+  const unsigned nt = (unsigned)tiles.size();
+  tmp.run([=] {
+    note_launch();
+    k_inv_upper<T><<<nt, 256, 0, st>>>(dut, dtl);
+  });
 }
 
 // ------------------------------------------------------------------ factor object
@@ -1482,6 +1596,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
     for (int c = 0; c < nc; ++c)
       if (L.cl[c].interior && n[c] > 0) I.push_back(c);
     if (!I.empty()) {
+      Deferred chain(tmp);
       std::vector<MatRef<T>> mats;
       std::vector<T*> Linv, Uinv;
       std::vector<const T*> nod;
@@ -1544,7 +1659,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       // triangular-times-dense products: m n k useful flops each (half of a full product)
       double gflops = 0;
       for (size_t q = 0; q < tasks.size(); ++q) gflops += 1.0 * tasks[q].m * (double)tasks[q].n * terms[q].k;
-      ev_begin(ev_gm[l]);
+      tmp.run([&, l] { ev_begin(ev_gm[l]); });
       launch_gemm(tmp, tasks, terms, st, "elim-YX");
       // Schur updates grouped by target block
       std::map<std::pair<int, int>, std::vector<int>> contrib;
@@ -1565,7 +1680,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
         for (int q = t0; q < (int)terms.size(); ++q) gflops += 2.0 * n[a] * (double)n[b] * terms[q].k;
       }
       launch_gemm(tmp, tasks, terms, st, "elim-schur");
-      ev_end(ev_gm[l]);
+      tmp.run([&, l] { ev_end(ev_gm[l]); });
       S.elim_gemm_flops += gflops;
       S.elim_gemm_launches += 2;
       if (l == D)
@@ -1590,6 +1705,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
     std::vector<std::vector<int>> nba(nc);
     for (auto& pr : L.after)
       if (pr.first != pr.second && n[pr.first] > 0 && n[pr.second] > 0) nba[pr.first].push_back(pr.second);
+    auto scale_chain = std::make_unique<Deferred>(tmp);
     std::vector<MatRef<T>> mats;
     std::vector<T*> SL, SU;
     std::vector<const T*> dsc;
@@ -1613,8 +1729,11 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
     if (!mats.empty()) {
       auto* dm = tmp.upload(mats);
       auto* dd = tmp.upload(dsc_mut);
-      note_launch();
-      k_diag_sqrt<T><<<(unsigned)mats.size(), 128, 0, st>>>(dm, dd, (int)mats.size());
+      const int nm = (int)mats.size();
+      tmp.run([=] {
+        note_launch();
+        k_diag_sqrt<T><<<(unsigned)nm, 128, 0, st>>>(dm, dd, nm);
+      });
     }
     batched_inverses(tmp, mats, SL, SU, dsc, st);
     {
@@ -1646,6 +1765,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       launch_gemm(tmp, t1, m1, st, "scale");
       launch_gemm(tmp, t2, m2, st, "scale");
     }
+    scale_chain.reset();
     mark(2);
     tick("c scale interfaces");
     // ================= 3. all Q first (Eq. 12): RRQR of [A_sn A_ns^T]
@@ -2184,16 +2304,23 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       }
       if (tmp.err) return SPAND_ERR_NOMEM;
       tick("g WY task lists");
+      Deferred chain(tmp);
       launch_gemm(tmp, gt, gm, st, "wy");
       if (!wy.empty()) {
         auto* dw = tmp.upload(wy);
-        note_launch();
-        k_wy_tinv<T><<<(unsigned)wy.size(), 256, 0, st>>>(dw);
+        const unsigned nw = (unsigned)wy.size();
+        tmp.run([=] {
+          note_launch();
+          k_wy_tinv<T><<<nw, 256, 0, st>>>(dw);
+        });
         // T = (T^-1)^-1 with the batched upper-triangular inverse
         batched_upper_inverse(tmp, tri, Tinv, st);
         auto* de = tmp.upload(eye_q);
-        note_launch();
-        k_eye<T><<<std::min<unsigned>((unsigned)eye_q.size(), 4096), 256, 0, st>>>(de, (int)eye_q.size());
+        const int ne = (int)eye_q.size();
+        tmp.run([=] {
+          note_launch();
+          k_eye<T><<<std::min<unsigned>((unsigned)ne, 4096), 256, 0, st>>>(de, ne);
+        });
       }
       launch_gemm(tmp, mt, mm, st, "wy");
       launch_gemm(tmp, qtk, qm, st, "wy");
@@ -2267,13 +2394,18 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
     }
     if (tmp.err) return SPAND_ERR_NOMEM;
     tick("j compress task lists");
+    auto merge_chain = std::make_unique<Deferred>(tmp);
     launch_gemm(tmp, t1, m1, st, "compress");
     launch_gemm(tmp, t2, m2, st, "compress");
     if (!eyes.empty()) {
       auto* de = tmp.upload(eyes);
-      note_launch();
-      k_eye<T><<<std::min<unsigned>((unsigned)eyes.size(), 1024), 128, 0, st>>>(de, (int)eyes.size());
+      const int ne = (int)eyes.size();
+      tmp.run([=] {
+        note_launch();
+        k_eye<T><<<std::min<unsigned>((unsigned)ne, 1024), 128, 0, st>>>(de, ne);
+      });
     }
+    merge_chain.reset();
     SPAND_CUDA_TRY(cudaGetLastError());
     tmp.free_all();
     lvmem.free_all();
@@ -2410,6 +2542,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
   const size_t es = sizeof(T);
   // sweeps of the clusters keep(l, c) selects (one system, or all of them)
   auto build_prog = [&](Program<T>& pg, auto keep) {
+  Deferred tables(pm);
   int64_t& apply_bytes = pg.bytes;
   gv_slots = 0;
   for (int tr = 0; tr < 2; ++tr) {
