@@ -2495,7 +2495,6 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
   int gv_slots = 0;                        // partial sums the program's longest phase keeps
   auto build = [&](std::vector<GvTask<T>>& tasks, std::vector<GvTerm<T>>& terms) -> Phase {
     Phase ph;
-    std::vector<GvTile> tiles;
     for (auto& tm : terms) {
       ph.kmax = std::max(ph.kmax, tm.k);
       if (tm.M && tm.trans) ph.trans = true;
@@ -2503,36 +2502,47 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
     size_t n32 = 0;
     for (auto& tk : tasks) n32 += (tk.m + GV_ROWS - 1) / GV_ROWS;
     if (!ph.trans && n32 >= GV_MANY) ph.groups = 2;
-    // chunks of every tile; tiles much longer than the phase's even share are cut
+    // chunks of every tile (a term without a triangle has as many in each tile of its task)
     int64_t all = 0;
     int jlo, jhi;
-    for (int t = 0; t < (int)tasks.size(); ++t)
+    std::vector<GvTile> tiles;
+    tiles.reserve(n32);
+    for (int t = 0; t < (int)tasks.size(); ++t) {
+      int full = 0;
+      bool tri = false;
+      for (int q = tasks[t].t0; q < tasks[t].t1; ++q) {
+        if (terms[q].M && terms[q].tri) tri = true;
+        else full += gv_chunks<1>(terms[q], 0, jlo, jhi);
+      }
       for (int r0 = 0; r0 < tasks[t].m; r0 += GV_ROWS * ph.groups) {
-        int n = 0;
-        for (int q = tasks[t].t0; q < tasks[t].t1; ++q)
-          n += ph.groups == 2 ? gv_chunks<2>(terms[q], r0, jlo, jhi) : gv_chunks<1>(terms[q], r0, jlo, jhi);
+        int n = full;
+        if (tri)
+          for (int q = tasks[t].t0; q < tasks[t].t1; ++q)
+            if (terms[q].M && terms[q].tri)
+              n += ph.groups == 2 ? gv_chunks<2>(terms[q], r0, jlo, jhi) : gv_chunks<1>(terms[q], r0, jlo, jhi);
         tiles.push_back({t, r0, 0, n, 0, 0, 1});
         all += n;
       }
+    }
     if (tiles.empty()) return ph;
+    // tiles longer than the phase's even share are cut; their pieces start first
     const int piece = std::max<int>(GV_PIECE, (int)(all / GV_MANY));
-    const size_t whole = tiles.size();
     int slots = 0;
-    for (size_t i = 0; i < whole; ++i) {
-      const GvTile tl = tiles[i];
+    std::vector<GvTile> cuts;
+    for (auto& tl : tiles) {
       const int ns = (tl.c1 + piece - 1) / piece;
       if (ns < 2) continue;
-      for (int g = 0; g < ns; ++g) {
-        const GvTile cut{tl.task, tl.r0, (int)((int64_t)tl.c1 * g / ns), (int)((int64_t)tl.c1 * (g + 1) / ns), slots, g, ns};
-        if (g == 0) tiles[i] = cut;
-        else tiles.push_back(cut);
-      }
+      for (int g = 0; g < ns; ++g)
+        cuts.push_back({tl.task, tl.r0, (int)((int64_t)tl.c1 * g / ns), (int)((int64_t)tl.c1 * (g + 1) / ns), slots, g, ns});
       slots += ns;
+      tl.nseg = 0;
+    }
+    if (slots) {
+      for (auto& tl : tiles)
+        if (tl.nseg) cuts.push_back(tl);
+      tiles.swap(cuts);
     }
     gv_slots = std::max(gv_slots, slots);
-    // the longest pieces start first
-    std::stable_sort(tiles.begin(), tiles.end(),
-                     [](const GvTile& a, const GvTile& b) { return a.c1 - a.c0 > b.c1 - b.c0; });
     upload3(pm, tasks, terms, tiles, ph.tasks, ph.terms, ph.tiles);
     ph.ntiles = (int)tiles.size();
     return ph;
