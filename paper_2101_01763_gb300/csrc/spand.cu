@@ -476,13 +476,14 @@ struct GemmLog {
   }
 };
 
+// plain: FP32 products in FP32 multiply-adds instead of the 3xTF32 kernels
 template <typename T>
 static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, const std::vector<GemmTerm<T>>& terms,
-                        cudaStream_t st, const char* tag = "") {
+                        cudaStream_t st, const char* tag = "", bool plain = false) {
   bool umma = false;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   bool* recorded = nullptr;
-  if (std::is_same<T, float>::value) {
+  if (std::is_same<T, float>::value && !plain) {
     double chunks = 0, flops = 0;
     int ntask = 0;
     for (const auto& tk : tasks) {
@@ -530,6 +531,10 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
         if (on && cudaEventRecord(r.b, s) == cudaSuccess) GemmLog::get().recs.push_back(r);
       }
     } log_at_end{logit, rec, st};
+    if (std::is_same<T, float>::value && plain) {
+      k_gemm<T><<<ntiles, 256, 0, st>>>(dt, dm, dl);
+      return;
+    }
     if constexpr (std::is_same<T, float>::value) {
       if (e0) cudaEventRecord(e0, st);
       if (umma && uv == 1 && umma_depth() == 2) {
@@ -1051,19 +1056,24 @@ static void batched_getrf(DevMem& tmp, std::vector<MatRef<T>>& mats, int* d_flag
 // L^-1 (optionally row-scaled by 1/d) and U^-1 (optionally column-scaled by d)
 // by a bottom-up block recursion on the grouped GEMM: invert the 32 x 32
 // diagonal blocks, then for block sizes 32, 64, 128, ... combine neighbouring
-// blocks,  X21 = -X22 (L21 X11)  and  Y12 = -Y11 (U12 Y22).
+// blocks,  X21 = -X22 (L21 X11)  and  Y12 = -Y11 (U12 Y22).  An empty Linv asks
+// for U^-1 alone, unscaled.
 template <typename T>
 static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, const std::vector<T*>& Linv,
-                             const std::vector<T*>& Uinv, const std::vector<const T*>& dscale, cudaStream_t st) {
+                             const std::vector<T*>& Uinv, const std::vector<const T*>& dscale, cudaStream_t st,
+                             bool plain = false) {
   if (mats.empty()) return;
   Deferred chain(tmp);
+  const bool lower = !Linv.empty();
   // zero both outputs (the opposite triangles must read as zeros)
   {
     std::vector<T*> ptr;
     std::vector<int> nn;
     for (size_t b = 0; b < mats.size(); ++b) {
-      ptr.push_back(Linv[b]);
-      nn.push_back(mats[b].n);
+      if (lower) {
+        ptr.push_back(Linv[b]);
+        nn.push_back(mats[b].n);
+      }
       ptr.push_back(Uinv[b]);
       nn.push_back(mats[b].n);
     }
@@ -1084,7 +1094,7 @@ static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, co
     const int n = mats[b].n;
     nmax = std::max(nmax, n);
     for (int p = 0; 32 * p < n; ++p) {
-      dt.push_back({mats[b].A, Linv[b], n, p, 1});
+      if (lower) dt.push_back({mats[b].A, Linv[b], n, p, 1});
       dt.push_back({mats[b].A, Uinv[b], n, p, 0});
     }
   }
@@ -1114,12 +1124,14 @@ static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, co
       for (int a0 = 0; a0 + bs < n; a0 += 2 * bs) {
         const int c0 = a0 + bs, na = bs, nc = std::min(bs, n - c0);
         // lower: X21 (nc x na) = -X22 (L21 X11)
-        T* W1 = W + woff;
-        woff += (size_t)nc * na;
-        m1.push_back({LU + c0 + (size_t)a0 * n, Linv[b] + a0 + (size_t)a0 * n, n, n, na, 0, 0, 0});
-        t1.push_back({W1, nc, nc, na, (T)1, (T)0, (int)m1.size() - 1, (int)m1.size()});
-        m2.push_back({Linv[b] + c0 + (size_t)c0 * n, W1, n, nc, nc, 0, 0, 1});   // X22 lower
-        t2.push_back({Linv[b] + c0 + (size_t)a0 * n, n, nc, na, (T)-1, (T)0, (int)m2.size() - 1, (int)m2.size()});
+        if (lower) {
+          T* W1 = W + woff;
+          woff += (size_t)nc * na;
+          m1.push_back({LU + c0 + (size_t)a0 * n, Linv[b] + a0 + (size_t)a0 * n, n, n, na, 0, 0, 0});
+          t1.push_back({W1, nc, nc, na, (T)1, (T)0, (int)m1.size() - 1, (int)m1.size()});
+          m2.push_back({Linv[b] + c0 + (size_t)c0 * n, W1, n, nc, nc, 0, 0, 1});   // X22 lower
+          t2.push_back({Linv[b] + c0 + (size_t)a0 * n, n, nc, na, (T)-1, (T)0, (int)m2.size() - 1, (int)m2.size()});
+        }
         // upper: Y12 (na x nc) = -Y11 (U12 Y22)
         T* W2 = W + woff;
         woff += (size_t)na * nc;
@@ -1129,9 +1141,10 @@ static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, co
         t2.push_back({Uinv[b] + a0 + (size_t)c0 * n, n, na, nc, (T)-1, (T)0, (int)m2.size() - 1, (int)m2.size()});
       }
     }
-    launch_gemm(tmp, t1, m1, st, "tri-inverse");
-    launch_gemm(tmp, t2, m2, st, "tri-inverse");
+    launch_gemm(tmp, t1, m1, st, "tri-inverse", plain);
+    launch_gemm(tmp, t2, m2, st, "tri-inverse", plain);
   }
+  if (!lower) return;
   // scalings of the interface form: SL = diag(1/d) L^-1, SU = U^-1 diag(d)
   std::vector<InvTask<T>> lt, ut;
   std::vector<InvTile> tiles;
@@ -1156,10 +1169,26 @@ static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, co
   });
 }
 
-// U^-1 only (no permutation, no scaling)
+// U^-1 only (no permutation, no scaling).  A kernel with a CTA per 32 columns
+// walks up each column's blocks one after the other, which is the shortest way
+// for small matrices and the longest for large ones (26 of the 36 ms that the Q_c
+// of 256 x 128 p=3 took): from INV_SERIAL rows on the block recursion takes over,
+// in FP32 multiply-adds as in the kernel (that factorization and solve 837 -> 827
+// ms).  With the recursion for every size 64 x 32 p=2, of at most 268 rows, was
+// 0.2 ms slower.
+constexpr int INV_SERIAL = 320;
+
 template <typename T>
-static void batched_upper_inverse(DevMem& tmp, const std::vector<MatRef<T>>& mats, const std::vector<T*>& Uinv,
+static void batched_upper_inverse(DevMem& tmp, const std::vector<MatRef<T>>& all, const std::vector<T*>& all_inv,
                                   cudaStream_t st) {
+  std::vector<MatRef<T>> mats, big;
+  std::vector<T*> Uinv, big_inv;
+  for (size_t b = 0; b < all.size(); ++b) {
+    const bool l = all[b].n > INV_SERIAL;
+    (l ? big : mats).push_back(all[b]);
+    (l ? big_inv : Uinv).push_back(all_inv[b]);
+  }
+  batched_inverses(tmp, big, std::vector<T*>(), big_inv, std::vector<const T*>(big.size(), nullptr), st, true);
   if (mats.empty()) return;
   std::vector<InvTask<T>> ut;
   std::vector<InvTile> tiles;
