@@ -344,6 +344,13 @@ static int umma_depth() {
   return d;
 }
 
+// k_gemm_umma's tiles are 128 wide where that covers at most a quarter more area
+// than tiles 64 wide and leaves each of 152 SMs its two CTAs.  Factorization and
+// solve of 256 x 128 p=3: all 64 wide 827 ms, this rule 815; a tenth more area and
+// no count 820.  64 x 32 p=2: 35.65, 35.39, 35.38 ms.
+constexpr double UM_WIDE_FILL = 1.25;
+constexpr long UM_WIDE_TILES = 2 * 152;
+
 // Online tuner for the choice of GEMM kernel (and with it the tile shape).
 // Launches are grouped by device, the average number of 32-wide k-chunks per
 // product (log2 bucket) and the logical flop count (log2 bucket).  The first
@@ -497,7 +504,15 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
     if (ntask > 0) umma = gemm_pick(chunks / ntask, flops, e0, e1, recorded) == 0;
   }
   const int uv = umma_variant();
-  const int BM = umma ? (uv == 2 ? U2_BM : UM_BM) : 64, BN = umma ? (uv == 2 ? U2_BN : UM_BN) : 64;
+  bool wide = false;
+  if (umma && uv == 1) {
+    long cnt[2] = {0, 0};   // tiles 64 and 128 wide
+    for (const auto& tk : tasks)
+      for (int w = 0; w < 2; ++w)
+        cnt[w] += (long)((tk.m + UM_BM - 1) / UM_BM) * ((tk.n + (64 << w) - 1) / (64 << w));
+    wide = 2 * cnt[1] <= UM_WIDE_FILL * cnt[0] && cnt[1] >= UM_WIDE_TILES;
+  }
+  const int BM = umma ? (uv == 2 ? U2_BM : UM_BM) : 64, BN = umma ? (uv == 2 ? U2_BN : wide ? 2 * UM_BN : UM_BN) : 64;
   std::vector<TileItem> tiles;
   for (int t = 0; t < (int)tasks.size(); ++t) {
     if (tasks[t].m <= 0 || tasks[t].n <= 0) continue;
@@ -537,14 +552,13 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
     }
     if constexpr (std::is_same<T, float>::value) {
       if (e0) cudaEventRecord(e0, st);
-      if (umma && uv == 1 && umma_depth() == 2) {
-        static std::atomic<uint64_t> attr{0};
-        once_per_device(attr, [] { set_dyn_smem((const void*)k_gemm_umma<2>, UM_SMEM_BYTES); });
-        k_gemm_umma<2><<<ntiles, 128, UM_SMEM_BYTES, st>>>(dt, dm, dl);
-      } else if (umma && uv == 1) {
-        static std::atomic<uint64_t> attr1{0};
-        once_per_device(attr1, [] { set_dyn_smem((const void*)k_gemm_umma<1>, UM_SMEM_BYTES); });
-        k_gemm_umma<1><<<ntiles, 128, UM_SMEM_BYTES, st>>>(dt, dm, dl);
+      if (umma && uv == 1) {
+        const bool deep = umma_depth() == 2;
+        auto kern = wide ? (deep ? k_gemm_umma<2, 128> : k_gemm_umma<1, 128>)
+                         : (deep ? k_gemm_umma<2, 64> : k_gemm_umma<1, 64>);
+        static std::atomic<uint64_t> attr[2];
+        once_per_device(attr[wide], [&] { set_dyn_smem((const void*)kern, um_smem_bytes(BN)); });
+        kern<<<ntiles, 2 * BN, um_smem_bytes(BN), st>>>(dt, dm, dl);
       } else if (umma && uv == 3) {
         static std::atomic<uint64_t> attr3{0};
         once_per_device(attr3, [] { set_dyn_smem((const void*)k_gemm_umma3, U3_SMEM_BYTES); });

@@ -1,19 +1,19 @@
 // Grouped FP32 GEMM on the 5th-generation tensor cores (tcgen05, sm_100 family).
 //
 // Same task / term / tile contract as k_gemm_tc (C = alpha * sum_t op(A_t) op(B_t)
-// + beta * C, column-major), on 128 x 64 output tiles:
-//  * 128 threads stage one 16-wide k-chunk of op(A) (128 x 16) and op(B)^T
-//    (64 x 16) in shared memory, split into TF32 high parts (rounded) and the
+// + beta * C, column-major), on output tiles of 128 x 64 or 128 x 128:
+//  * 128 (256) threads stage one 16-wide k-chunk of op(A) (128 x 16) and op(B)^T
+//    (64 or 128 x 16) in shared memory, split into TF32 high parts (rounded) and the
 //    exact FP32 remainders (of which the tensor core reads the top 19 bits),
 //    in the K-major "core matrix" layout the MMA reads without swizzling
 //    (8 rows x 16 bytes per core matrix);
 //  * one thread issues tcgen05.mma.kind::tf32 with the accumulator in tensor
-//    memory (128 lanes x 64 FP32 columns): hi*lo + lo*hi + hi*hi per 8-wide
+//    memory (128 lanes x 64 or 128 FP32 columns): hi*lo + lo*hi + hi*hi per 8-wide
 //    k-step (error-compensated 3xTF32, about FP32 accuracy), and commits the
 //    chunk to an mbarrier of its stage; two stages alternate so the staging
 //    of chunk i+1 overlaps the MMAs of chunk i;
 //  * the epilogue reads the accumulator with tcgen05.ld (warp w owns lanes
-//    32w..32w+31 = rows of the tile) and applies alpha / beta.
+//    32 (w % 4) .. + 31 = rows of the tile, and 64 columns) and applies alpha / beta.
 // Every mbarrier wait is bounded; on timeout the CTA sets g_umma_fail (read by
 // the host after the factorization), skips its epilogue and frees its tensor
 // memory.
@@ -27,11 +27,10 @@ namespace spand {
 constexpr int UM_BM = 128, UM_BN = 64, UM_BK = 16;
 constexpr int UM_BH = UM_BK / 2;          // k values of a B column one thread stages
 constexpr int UM_SBO = 8 * UM_BK * 4;     // bytes between 8-row groups of a K-major operand
-constexpr int UM_TMEM_COLS = 64;
-// bytes of one operand stage: A hi, A lo (128 x 32 x 4), B hi, B lo (64 x 32 x 4)
-constexpr int UM_A_BYTES = UM_BM * UM_BK * 4, UM_B_BYTES = UM_BN * UM_BK * 4;
-constexpr int UM_STAGE_BYTES = 2 * UM_A_BYTES + 2 * UM_B_BYTES;
-constexpr int UM_SMEM_BYTES = 2 * UM_STAGE_BYTES + 1024;   // two stages + alignment slack
+constexpr int UM_A_BYTES = UM_BM * UM_BK * 4;
+// one operand stage: A hi, A lo (128 x 16 x 4 bytes), B hi, B lo (bn x 16 x 4 bytes)
+__host__ __device__ constexpr int um_stage_bytes(int bn) { return 2 * UM_A_BYTES + 2 * bn * UM_BK * 4; }
+__host__ __device__ constexpr int um_smem_bytes(int bn) { return 2 * um_stage_bytes(bn) + 1024; }   // two stages + alignment slack
 
 __device__ inline uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -46,9 +45,9 @@ __device__ inline uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) 
   return d;                                     // base offset 0, relative LBO, no swizzle
 }
 
-// instruction descriptor: D = F32, A = B = TF32, both K-major, M = 128, N = 64
-__host__ __device__ constexpr uint32_t umma_idesc_tf32() {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(UM_BN >> 3) << 17) | ((uint32_t)(UM_BM >> 4) << 24);
+// instruction descriptor: D = F32, A = B = TF32, both K-major, M = 128, N = bn
+__host__ __device__ constexpr uint32_t umma_idesc_tf32(int bn = UM_BN) {
+  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(UM_BM >> 4) << 24);
 }
 
 // byte offset of element (r, k) of a K-major operand of 32-wide k-chunks:
@@ -77,9 +76,17 @@ __device__ inline bool mbar_wait(uint32_t bar, uint32_t parity) {
 
 __device__ int g_umma_fail;   // set when an MMA completion wait ran out of time
 
-template <int DEPTH>
-__global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tasks, const GemmTerm<float>* terms,
+// BN = 64 on 128 threads or 128 on 256.  The kernel is bound by the instructions
+// that split the operands, a per-tile cost that grows with BM + BN against BM BN
+// products: the wide tile issues a quarter fewer per product, the narrow one
+// wastes less on small outputs (launch_gemm picks by the tiles' fill).
+template <int DEPTH, int BN>
+__global__ void __launch_bounds__(2 * BN, BN == 64 ? 4 : 2) k_gemm_umma(const GemmTask<float>* tasks, const GemmTerm<float>* terms,
                                                       const TileItem* tiles) {
+  constexpr int NT = 2 * BN;                    // threads
+  constexpr int NA = UM_BM * UM_BK / NT;        // values of A a thread stages per chunk (8 of B)
+  constexpr int KS = NT / 4;                    // rows between a thread's pieces of an operand stored along k
+  constexpr int B_BYTES = BN * UM_BK * 4, STAGE_BYTES = um_stage_bytes(BN);
   extern __shared__ unsigned char um_raw[];
   __shared__ uint64_t mbar[2];
   __shared__ uint32_t tmem_base;
@@ -88,12 +95,12 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
   unsigned char* um = um_raw + ((1024 - (smem_u32(um_raw) & 1023)) & 1023);
   const TileItem it = tiles[blockIdx.x];
   const GemmTask<float> tk = tasks[it.task];
-  const int i0 = it.tm * UM_BM, j0 = it.tn * UM_BN;
+  const int i0 = it.tm * UM_BM, j0 = it.tn * BN;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                 "r"(UM_TMEM_COLS));
+                 "r"(BN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
@@ -111,7 +118,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
   // (pf_t, pf_l) is the next chunk to load
   int nch = 0;
   for (int t = tk.t0; t < tk.t1; ++t) {
-    const int kl = term_klim(terms[t], i0, j0, UM_BM, UM_BN);
+    const int kl = term_klim(terms[t], i0, j0, UM_BM, BN);
     if (kl > 0) nch += (kl + UM_BK - 1) / UM_BK;
   }
   // the term being loaded stays in registers (ct, its k limit ct_kl): a
@@ -122,7 +129,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
   auto seek = [&]() {     // first term from pf_t on with a non-empty k range
     for (; pf_t < tk.t1; ++pf_t) {
       ct = terms[pf_t];
-      ct_kl = term_klim(ct, i0, j0, UM_BM, UM_BN);
+      ct_kl = term_klim(ct, i0, j0, UM_BM, BN);
       if (ct_kl > 0) break;
     }
   };
@@ -138,17 +145,18 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
   int item = 0;
   bool failed = false;
   // operand values of one k-chunk held in registers as pieces of 4 consecutive
-  // k of one row: 4 pieces of op(A) (128 x UM_BK) and 2 of op(B)^T (64 x UM_BK).
+  // k of one row: NA / 4 pieces of op(A) (128 x UM_BK) and 2 of op(B)^T (BN x UM_BK).
   // An operand stored along k is read 8 rows x 64 bytes per warp instruction
-  // (piece q of lane l: row kr + 32 q, k offset kk); one stored along m (n)
+  // (piece q of lane l: row kr + KS q, k offset kk); one stored along m (n)
   // keeps a row (column) per thread and reads its k values one at a time, 32
   // consecutive rows per warp instruction.  DEPTH register sets: the loads of
   // chunk i + DEPTH are issued right after the MMAs of chunk i, so their
   // latency overlaps the staging and tensor-core work of DEPTH chunks.
   const int kr = 8 * warp + (lane & 7), kk = 4 * (lane >> 3);
-  const int c = tid & 63, half = tid >> 6;
-  const uint64_t desc0 = umma_desc(smem_u32(um), 128, UM_SBO), desc1 = umma_desc(smem_u32(um + UM_STAGE_BYTES), 128, UM_SBO);
-  auto load_chunk = [&](int l_, float (&x)[UM_BK], float (&y)[UM_BH], bool& a_kc, bool& b_kc) {
+  const int c = tid & (BN - 1), half = tid / BN;
+  const int ar = tid & (UM_BM - 1), ak = tid / UM_BM * NA;   // row and first k of A stored along m
+  const uint64_t desc0 = umma_desc(smem_u32(um), 128, UM_SBO), desc1 = umma_desc(smem_u32(um + STAGE_BYTES), 128, UM_SBO);
+  auto load_chunk = [&](int l_, float (&x)[NA], float (&y)[UM_BH], bool& a_kc, bool& b_kc) {
     const GemmTerm<float>& tm = ct;
     a_kc = tm.ta != 0;
     b_kc = tm.tb == 0;
@@ -156,8 +164,8 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
       const int gl = l_ + kk;
       const bool vec = ((tm.lda & 3) == 0) && ((reinterpret_cast<uintptr_t>(tm.A) & 15) == 0) && gl + 4 <= tm.k;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int gi = i0 + kr + 32 * q;
+      for (int q = 0; q < NA / 4; ++q) {
+        const int gi = i0 + kr + KS * q;
         if (vec) {
           const float4 f = gi < tk.m ? *reinterpret_cast<const float4*>(tm.A + gl + (size_t)gi * tm.lda)
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -172,18 +180,18 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
         }
       }
     } else {
-      const int gi = i0 + tid;
-      const float* pa = tm.A + gi + (size_t)l_ * tm.lda;
-      const int nk = gi < tk.m ? tm.k - l_ : 0;     // k values left in this row
+      const int gi = i0 + ar, ka = l_ + ak;
+      const float* pa = tm.A + gi + (size_t)ka * tm.lda;
+      const int nk = gi < tk.m ? tm.k - ka : 0;     // k values left in this row
 #pragma unroll
-      for (int e = 0; e < UM_BK; ++e) x[e] = e < nk ? pa[e * tm.lda] : 0.f;
+      for (int e = 0; e < NA; ++e) x[e] = e < nk ? pa[e * tm.lda] : 0.f;
     }
     if (b_kc) {
       const int gl = l_ + kk;
       const bool vec = ((tm.ldb & 3) == 0) && ((reinterpret_cast<uintptr_t>(tm.B) & 15) == 0) && gl + 4 <= tm.k;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        const int gj = j0 + kr + 32 * q;
+        const int gj = j0 + kr + KS * q;
         if (vec) {
           const float4 f = gj < tk.n ? *reinterpret_cast<const float4*>(tm.B + gl + (size_t)gj * tm.ldb)
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -206,9 +214,9 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
     }
   };
   // stage chunk `item` from registers and issue its MMAs; false on a timed-out wait
-  auto process = [&](const float (&x)[UM_BK], const float (&y)[UM_BH], bool a_kc, bool b_kc) -> bool {
+  auto process = [&](const float (&x)[NA], const float (&y)[UM_BH], bool a_kc, bool b_kc) -> bool {
     const int s = item & 1;
-    unsigned char* st = um + s * UM_STAGE_BYTES;
+    unsigned char* st = um + s * STAGE_BYTES;
     if (item >= 2) {
       // the MMAs that read this stage two chunks ago must be done; one thread
       // polls, the others wait at the barrier, and the outcome is uniform
@@ -218,7 +226,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
     // ---- split the chunk's values into TF32 hi / lo in the core-matrix layout
     {
 #pragma unroll
-      for (int kq = 0; kq < UM_BK; kq += 4) {
+      for (int kq = 0; kq < NA; kq += 4) {
         uint4 hi, lo;
         hi.x = to_tf32(x[kq]);
         hi.y = to_tf32(x[kq + 1]);
@@ -228,7 +236,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
         lo.y = __float_as_uint(x[kq + 1] - __uint_as_float(hi.y));
         lo.z = __float_as_uint(x[kq + 2] - __uint_as_float(hi.z));
         lo.w = __float_as_uint(x[kq + 3] - __uint_as_float(hi.w));
-        const uint32_t off = a_kc ? umma_off_bk(kr + 8 * kq, kk) : umma_off_bk(tid, kq);   // piece kq / 4
+        const uint32_t off = a_kc ? umma_off_bk(kr + KS / 4 * kq, kk) : umma_off_bk(ar, ak + kq);   // piece kq / 4
         *reinterpret_cast<uint4*>(st + off) = hi;
         *reinterpret_cast<uint4*>(st + UM_A_BYTES + off) = lo;
       }
@@ -243,9 +251,9 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
         lo.y = __float_as_uint(y[kq + 1] - __uint_as_float(hi.y));
         lo.z = __float_as_uint(y[kq + 2] - __uint_as_float(hi.z));
         lo.w = __float_as_uint(y[kq + 3] - __uint_as_float(hi.w));
-        const uint32_t off = b_kc ? umma_off_bk(kr + 8 * kq, kk) : umma_off_bk(c, half * UM_BH + kq);
+        const uint32_t off = b_kc ? umma_off_bk(kr + KS / 4 * kq, kk) : umma_off_bk(c, half * UM_BH + kq);
         *reinterpret_cast<uint4*>(st + 2 * UM_A_BYTES + off) = hi;
-        *reinterpret_cast<uint4*>(st + 2 * UM_A_BYTES + UM_B_BYTES + off) = lo;
+        *reinterpret_cast<uint4*>(st + 2 * UM_A_BYTES + B_BYTES + off) = lo;
       }
     }
     // the generic-proxy stores must be visible to the tensor core (async proxy)
@@ -253,7 +261,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
     __syncthreads();
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint32_t idesc = umma_idesc_tf32();
+      const uint32_t idesc = umma_idesc_tf32(BN);
       const uint64_t d0 = s ? desc1 : desc0;   // descriptor of the stage's A hi part
 #pragma unroll
       for (int ks = 0; ks < UM_BK / 8; ++ks) {
@@ -261,7 +269,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
         // addresses are in 16-byte units in the low bits
         const uint64_t ko = (uint64_t)(ks * 256) >> 4;
         const uint64_t dah = d0 + ko, dal = d0 + ko + (UM_A_BYTES >> 4);
-        const uint64_t dbh = d0 + ko + ((2 * UM_A_BYTES) >> 4), dbl = d0 + ko + ((2 * UM_A_BYTES + UM_B_BYTES) >> 4);
+        const uint64_t dbh = d0 + ko + ((2 * UM_A_BYTES) >> 4), dbl = d0 + ko + ((2 * UM_A_BYTES + B_BYTES) >> 4);
         const uint32_t acc0 = (item > 0 || ks > 0) ? 1u : 0u;
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(
@@ -282,7 +290,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
     ++item;
     return true;
   };
-  float x0[UM_BK], y0[UM_BH], x1[UM_BK], y1[UM_BH];
+  float x0[NA], y0[UM_BH], x1[NA], y1[UM_BH];
   bool ak0 = false, bk0 = false, ak1 = false, bk1 = false;
   if (pf_t < tk.t1) {
     load_chunk(pf_l, x0, y0, ak0, bk0);
@@ -323,13 +331,14 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
   if (s_fail) {
     if (tid == 0) atomicOr(&g_umma_fail, 1);
   } else {
-    // ---- epilogue: warp w holds rows 32w..32w+31 of the tile, 64 columns each
-    const int row = warp * 32 + lane, gi = i0 + row;
+    // ---- epilogue: warp w reads rows 32 (w % 4) .. + 31 of the tile, 64 columns
+    const int row = (warp & 3) * 32 + lane, gi = i0 + row;
 #pragma unroll
-    for (int cb = 0; cb < UM_BN; cb += 16) {
+    for (int cc = 0; cc < 64; cc += 16) {
+      const int cb = (warp >> 2) * 64 + cc;
       uint32_t v[16];
       if (item > 0) {
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cb;
+        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)cb;
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
@@ -359,7 +368,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm_umma(const GemmTask<float>* tas
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(UM_TMEM_COLS));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
   }
 }
 
