@@ -400,11 +400,11 @@ def rooflines(sg, torch, W, fst, flush, stream, peaks_):
     # the GEMMs run inside a seconds-long factorization: the sustained bf16 figure
     bf16 = float(pk.get("bf16_tflops_sustained", pk.get("bf16_tflops", PEAKS_FALLBACK["bf16_tflops"])))
     tf32_peak = bf16 * (1.1 / 2.25)          # nominal TF32 : BF16 dense ratio
-    # rank-revealing QR of the sparsification (k_qrcp_stream); one "launch" = the
-    # RRQR phase of one level (its kernels between two events on the factor's
-    # stream).  Bound by the traffic of the live columns: the kernel counts the
-    # bytes its column passes move (each live column read and written once per
-    # pivot step).  The method's own work, 4 (n-k)(c-k) flops per pivot step
+    # rank-revealing QR of the sparsification (k_qrcp_stream_group / _solo); one
+    # "launch" = the RRQR phase of one level (its kernels between two events on the
+    # factor's stream).  The kernels count the bytes their column passes move (an
+    # active column read and written once per pivot step, a waiting one once per
+    # bring-up); the time goes to the pivot steps' latency and the bring-ups.  The method's own work, 4 (n-k)(c-k) flops per pivot step
     # (reflector dot products and update over every column), is reported beside.
     nl = max(1, fst["rrqr_launches"])
     rr_ms = fst["t_rrqr_ms"] / nl
@@ -445,11 +445,12 @@ def rooflines(sg, torch, W, fst, flush, stream, peaks_):
     t_spmv = statistics.mean(sp_ms)
     sp_bytes = W.A.nnzb * W.A.B * W.A.B * 8 + 2 * W.A.K * W.A.B * 8
     sp_ach = sp_bytes / (t_spmv * 1e-3) / 1e9
-    rr = {"kernel": "k_qrcp_stream (column-pivoted Householder QR of the interface sparsification, W streamed "
+    rr = {"kernel": "k_qrcp_stream_group / _solo (column-pivoted Householder QR of the interface sparsification, W streamed "
                     "from L2/HBM; one launch = the RRQR phase of one level)",
           "bound": "hbm", "achieved": rr_ach, "peak": hbm, "unit": "GB/s", "frac": rr_ach / hbm, "traffic": None,
           "peak_kind": f"{pk_kind} hbm_gbs", "bytes_per_launch": rr_bytes, "ms_per_launch": rr_ms,
-          "bytes_rule": "2 (n-k) m_k x 4 per pivot step k, m_k = live columns (counted by the kernel)",
+          "bytes_rule": "2 (n-k) x 4 per column and pass: active columns per pivot step, waiting ones per "
+                        "bring-up (counted by the kernel)",
           "method_flops_per_launch": rr_flops,
           "method_tflops": rr_flops / (rr_ms * 1e-3) / 1e12 if rr_ms > 0 else 0.0,
           "method_flops_rule": "4 (n-k)(c-k) per pivot step k over every column"}

@@ -6,8 +6,8 @@
 // norm never grows, so the norm a column had when it was last touched bounds
 // its norm now.  The factorization therefore runs in bands: with m the largest
 // bound of the remaining columns, the columns whose bound is at least m / f are
-// brought up to date (the reflectors they have missed are applied one after the
-// other while the column stays in registers, and its norm is recomputed); those
+// brought up to date (the reflectors they have missed are applied in blocks of
+// QRS_NB while the column stays in shared memory, and its norm is recomputed); those
 // still at or above m / f are the band's active columns.  Pivot steps then
 // touch the active columns alone, until the largest active norm falls below
 // m / f: until then no other column can be the pivot.  A column that falls
@@ -22,8 +22,8 @@
 // of that discretisation the band form touches 3 to 7 % of those column-steps at
 // f = 1.5 to 2 and 1.4 % more for the bring-ups.  What is left is the arithmetic
 // of the bring-ups (4 flops per element and missed reflector) and the latency of
-// the r sequential pivot steps: 90 ms at the leaf level, 223 ms in all (C2 size,
-// 64 x 32 p=2: 11.3 ms before, 9.0 ms now; FP64 there 64 and 38 ms).
+// the r sequential pivot steps: 90 ms at the leaf level, 223 ms in all (64 x 32
+// p=2: 11.3 ms before, 9.0 ms now; FP64 there 64 and 38 ms).
 //
 // Layout and work split.  W is column-major (column j at W + j*ldw, ldw a
 // multiple of 16 bytes), V has its columns on 128-byte lines (ldv), so no line
