@@ -2568,7 +2568,7 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       }
     }
     if (tiles.empty()) return ph;
-    // tiles longer than the phase's even share are cut; their pieces start first
+    // tiles longer than the phase's even share are cut
     const int piece = std::max<int>(GV_PIECE, (int)(all / GV_MANY));
     int slots = 0;
     std::vector<GvTile> cuts;
@@ -2586,6 +2586,16 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       tiles.swap(cuts);
     }
     gv_slots = std::max(gv_slots, slots);
+    // the longest first (a counting sort; in the tasks' order 192 x 96 p=3 solves
+    // in 116.5 ms, in this one in 111.5)
+    int most = 0;
+    for (const auto& tl : tiles) most = std::max(most, tl.c1 - tl.c0);
+    std::vector<int> at(most + 2, 0);
+    for (const auto& tl : tiles) ++at[most - (tl.c1 - tl.c0) + 1];
+    for (int l = 0; l <= most; ++l) at[l + 1] += at[l];
+    cuts.resize(tiles.size());
+    for (const auto& tl : tiles) cuts[at[most - (tl.c1 - tl.c0)]++] = tl;
+    tiles.swap(cuts);
     upload3(pm, tasks, terms, tiles, ph.tasks, ph.terms, ph.tiles);
     ph.ntiles = (int)tiles.size();
     return ph;
