@@ -159,7 +159,11 @@ static int spmv_launch(const bsr_matrix* A, const TX* x, double* y, int transpos
   if (!transpose)
     k_bsr_spmv<TX><<<(unsigned)((n + 31) / 32), 256, 0, st>>>(A->K, A->B, A->row_ptr, A->col, A->val, x, y, sa,
                                                                    a1, u1, a2, u2);
-  else if ((A->B == 16 || A->B == 36 || A->B == 64) && (reinterpret_cast<uintptr_t>(A->val) & 15) == 0) {
+  else if ((A->B == 64 || (A->B == 36 && A->K <= 1024) || (A->B == 16 && A->K <= 4096)) &&
+           (reinterpret_cast<uintptr_t>(A->val) & 15) == 0) {
+    // small blocks leave lanes idle: past these K a thread per column is as fast or faster (us, CTA per row
+    // against thread per column: B = 36, K = 660 20 and 27, 2,048 47 and 41, 32,768 648 and 520; B = 16, K = 2,048
+    // 16 and 19, 8,192 49 and 49, 32,768 193 and 184; B = 64 84 and 182 at 2,048)
     auto k = A->B == 16 ? k_bsr_spmv_tb<TX, 16, 8> : A->B == 36 ? k_bsr_spmv_tb<TX, 36, 9> : k_bsr_spmv_tb<TX, 64, 16>;
     k<<<(unsigned)A->K, 256, 0, st>>>(A->K, A->row_ptr, A->col, A->val, x, y, sa, a1, u1, a2, u2);
   } else                            // other block sizes, or values not on a 16-byte boundary
