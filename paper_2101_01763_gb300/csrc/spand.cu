@@ -33,6 +33,7 @@
 #include "dense.cuh"
 #include "qrcp_stream.cuh"
 #include "gemm_split.cuh"
+#include "gemm_tuner.h"
 #include "gemv.cuh"
 #include "umma.cuh"
 #include "umma2.cuh"
@@ -351,93 +352,18 @@ static int umma_depth() {
 constexpr double UM_WIDE_FILL = 1.25;
 constexpr long UM_WIDE_TILES = 2 * 152;
 
-// Online tuner for the choice of GEMM kernel (and with it the tile shape).
-// Launches are grouped by device, the average number of 32-wide k-chunks per
-// product (log2 bucket) and the logical flop count (log2 bucket).  The first
-// launches of a class run each candidate once between two events; once both
-// timings have completed (checked without waiting, at a later launch of the
-// class) the candidate with the lower time per flop is used for the class for
-// the rest of the process.  Until then -- and whenever a measurement is still
-// in flight -- the rule "tcgen05 from four k-chunks per product on" decides.
-// Either kernel computes the same products; only FP32 rounding order differs.
-struct GemmTuner {
-  struct Entry {
-    int choice = -1;                 // decided: 0 tcgen05, 1 mma.sync
-    bool pending[2] = {false, false};
-    bool recorded[2] = {false, false};   // both events are on the stream
-    bool done[2] = {false, false};
-    double per_flop[2] = {0, 0};
-    double flops[2] = {0, 0};
-    cudaEvent_t ev[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-  };
-  std::mutex mu;
-  std::map<std::tuple<int, int, int>, Entry> table;
-  static GemmTuner& get() {
-    static GemmTuner* t = new GemmTuner();   // process lifetime
-    return *t;
-  }
-};
-
 // returns the kernel (0 tcgen05, 1 mma.sync) and, when this launch is to be
-// timed, the two events to record around it and the flag to set then
-static int gemm_pick(double avg_chunks, double flops, cudaEvent_t& e0, cudaEvent_t& e1, bool*& recorded) {
-  e0 = e1 = nullptr;
-  recorded = nullptr;
-  const int rule = avg_chunks >= 4.0 ? 0 : 1;
+// timed, its trial
+static int gemm_pick(double avg_chunks, double flops, std::shared_ptr<GemmTuner::Trial>& trial) {
   if (gemm_mode() == 1) return 0;
   if (gemm_mode() == 2) return 1;
   int dev = 0;
   cudaGetDevice(&dev);
-  const int cb = std::min(6, (int)std::floor(std::log2(std::max(1.0, avg_chunks))));
-  const int fb = std::min(12, (int)std::floor(std::log2(std::max(1.0, flops / 1e7))));
-  GemmTuner& T = GemmTuner::get();
-  std::lock_guard<std::mutex> g(T.mu);
-  GemmTuner::Entry& E = T.table[std::make_tuple(dev, cb, fb)];
-  if (E.choice >= 0) return E.choice;
-  for (int c = 0; c < 2; ++c)
-    if (E.pending[c] && E.recorded[c] && !E.done[c]) {
-      const cudaError_t q = cudaEventQuery(E.ev[c][1]);
-      if (q == cudaSuccess) {
-        float ms = 0.f;
-        if (cudaEventElapsedTime(&ms, E.ev[c][0], E.ev[c][1]) == cudaSuccess && E.flops[c] > 0) {
-          E.per_flop[c] = ms / E.flops[c];
-          E.done[c] = true;
-        }
-        E.pending[c] = E.recorded[c] = false;
-      } else if (q == cudaErrorNotReady && cudaPeekAtLastError() == cudaErrorNotReady) {
-        cudaGetLastError();          // a not-ready query is not an error of ours
-      }
-    }
-  if (E.done[0] && E.done[1]) {
-    E.choice = E.per_flop[0] <= E.per_flop[1] ? 0 : 1;
-    for (auto& pr : E.ev)
-      for (auto& e : pr)
-        if (e) cudaEventDestroy(e);
-    static const bool dbg = [] {
-      const char* v = std::getenv("SPAND_DEBUG");
-      return v && v[0] == '1';
-    }();
-    if (dbg)
-      std::fprintf(stderr, "spand: GEMM class (k-chunks 2^%d, flops 2^%d x 1e7): tcgen05 %.3g, mma.sync %.3g ms/GF -> %s\n",
-                   cb, fb, E.per_flop[0] * 1e9, E.per_flop[1] * 1e9, E.choice == 0 ? "tcgen05" : "mma.sync");
-    return E.choice;
-  }
-  for (int c = 0; c < 2; ++c)
-    if (!E.done[c] && !E.pending[c]) {
-      if (!E.ev[c][0]) {
-        if (cudaEventCreate(&E.ev[c][0]) != cudaSuccess || cudaEventCreate(&E.ev[c][1]) != cudaSuccess) {
-          cudaGetLastError();
-          return rule;
-        }
-      }
-      E.pending[c] = true;
-      E.flops[c] = flops;
-      e0 = E.ev[c][0];
-      e1 = E.ev[c][1];
-      recorded = &E.recorded[c];
-      return c;
-    }
-  return rule;                       // both measurements still in flight
+  static const bool dbg = [] {
+    const char* v = std::getenv("SPAND_DEBUG");
+    return v && v[0] == '1';
+  }();
+  return GemmTuner::get().pick(dev, avg_chunks, flops, dbg, trial);
 }
 
 // SPAND_DEBUG=3: CUDA-event time, logical flops and kernel of every grouped
@@ -488,8 +414,7 @@ template <typename T>
 static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, const std::vector<GemmTerm<T>>& terms,
                         cudaStream_t st, const char* tag = "", bool plain = false) {
   bool umma = false;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  bool* recorded = nullptr;
+  std::shared_ptr<GemmTuner::Trial> trial;
   if (std::is_same<T, float>::value && !plain) {
     double chunks = 0, flops = 0;
     int ntask = 0;
@@ -501,7 +426,7 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
       }
       ++ntask;
     }
-    if (ntask > 0) umma = gemm_pick(chunks / ntask, flops, e0, e1, recorded) == 0;
+    if (ntask > 0) umma = gemm_pick(chunks / ntask, flops, trial) == 0;
   }
   const int uv = umma_variant();
   bool wide = false;
@@ -551,7 +476,7 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
       return;
     }
     if constexpr (std::is_same<T, float>::value) {
-      if (e0) cudaEventRecord(e0, st);
+      if (trial) trial->begin(st);
       if (umma && uv == 1) {
         const bool deep = umma_depth() == 2;
         auto kern = wide ? (deep ? k_gemm_umma<2, 128> : k_gemm_umma<1, 128>)
@@ -570,10 +495,7 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
       } else {
         k_gemm_tc<3><<<ntiles, 128, 0, st>>>(dt, dm, dl);   // 3xTF32 on mma.sync
       }
-      if (e1 && cudaEventRecord(e1, st) == cudaSuccess) {
-        std::lock_guard<std::mutex> g(GemmTuner::get().mu);
-        *recorded = true;
-      }
+      if (trial) trial->end(st);
     } else {
       // the split kernel works in 64-wide chunks of k: below 48 values of k per
       // product on average (the 32-wide LU updates) its chunks are mostly padding
