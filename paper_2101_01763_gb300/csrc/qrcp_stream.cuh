@@ -73,7 +73,6 @@ struct Vec16<float> {
   using V = float4;
   static constexpr int W = 4;
   __device__ static inline V load(const float* p) { return *reinterpret_cast<const float4*>(p); }
-  __device__ static inline V ldcg(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
   __device__ static inline void store(float* p, const V& v) { *reinterpret_cast<float4*>(p) = v; }
   __device__ static inline float get(const V& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
   __device__ static inline void set(V& v, int i, float a) {
@@ -88,7 +87,6 @@ struct Vec16<double> {
   using V = double2;
   static constexpr int W = 2;
   __device__ static inline V load(const double* p) { return *reinterpret_cast<const double2*>(p); }
-  __device__ static inline V ldcg(const double* p) { return __ldcg(reinterpret_cast<const double2*>(p)); }
   __device__ static inline void store(double* p, const V& v) { *reinterpret_cast<double2*>(p) = v; }
   __device__ static inline double get(const V& v, int i) { return i == 0 ? v.x : v.y; }
   __device__ static inline void set(V& v, int i, double a) {

@@ -435,7 +435,7 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
     for (const auto& tk : tasks)
       for (int w = 0; w < 2; ++w)
         cnt[w] += (long)((tk.m + UM_BM - 1) / UM_BM) * ((tk.n + (64 << w) - 1) / (64 << w));
-    wide = 2 * cnt[1] <= UM_WIDE_FILL * cnt[0] && cnt[1] >= UM_WIDE_TILES;
+    wide = umma_depth() == 1 && 2 * cnt[1] <= UM_WIDE_FILL * cnt[0] && cnt[1] >= UM_WIDE_TILES;
   }
   const int BM = umma ? (uv == 2 ? U2_BM : UM_BM) : 64, BN = umma ? (uv == 2 ? U2_BN : wide ? 2 * UM_BN : UM_BN) : 64;
   std::vector<TileItem> tiles;
@@ -478,9 +478,7 @@ static void launch_gemm(DevMem& tmp, const std::vector<GemmTask<T>>& tasks, cons
     if constexpr (std::is_same<T, float>::value) {
       if (trial) trial->begin(st);
       if (umma && uv == 1) {
-        const bool deep = umma_depth() == 2;
-        auto kern = wide ? (deep ? k_gemm_umma<2, 128> : k_gemm_umma<1, 128>)
-                         : (deep ? k_gemm_umma<2, 64> : k_gemm_umma<1, 64>);
+        auto kern = wide ? k_gemm_umma<1, 128> : umma_depth() == 2 ? k_gemm_umma<2, 64> : k_gemm_umma<1, 64>;
         static std::atomic<uint64_t> attr[2];
         once_per_device(attr[wide], [&] { set_dyn_smem((const void*)kern, um_smem_bytes(BN)); });
         kern<<<ntiles, 2 * BN, um_smem_bytes(BN), st>>>(dt, dm, dl);
@@ -2242,7 +2240,6 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
       std::vector<WyTask<T>> wy;
       std::vector<MatRef<T>> tri;
       std::vector<T*> Tinv;
-      std::vector<const T*> nod;
       std::vector<EyeTask<T>> eye_q;
       for (size_t q = 0; q < qt.size(); ++q) {
         const int r = rank[q], nn = qt[q].n;
@@ -2260,7 +2257,6 @@ static int factor_impl(const Plan& P, const bsr_matrix* const* As, double eps, i
         mr.perm = nullptr;
         tri.push_back(mr);
         Tinv.push_back(Tm);
-        nod.push_back(nullptr);
         mm.push_back({Tm, qt[q].V, r, ldv[q], r, 0, 1, 0});
         mt.push_back({M, r, r, r, (T)1, (T)0, (int)mm.size() - 1, (int)mm.size()});
         eye_q.push_back({qt[q].Q, nn, r, nn});     // Q_c = [I_r; 0] before the update below
