@@ -241,8 +241,7 @@ __global__ void __launch_bounds__(256) k_getrf_panel(const MatRef<T>* mats, int 
 // at most 2 jb rows move).  rec[0] = count, rec[1..] = pos, rec[1 + 2 LU_NB..]
 // = src.  One warp: lane l holds the panel's own row l and the l-th other row
 // that moves, so an interchange is a ballot and two shuffles.  (One thread with
-// the lists in local memory took longer than the panel's 32 columns: 60 of 93 us
-// per panel at 64 x 32 p=2.)
+// the lists in local memory took 13 us of a panel of 64 rows, 21 at 1,152.)
 __device__ inline void lu_record_interchanges(int* rec, const int* piv_loc, int jb) {
   const int lane = threadIdx.x & 31;
   int src0 = lane, pos1 = -1, src1 = -1, ne = 0;
@@ -286,10 +285,15 @@ __device__ inline void lu_record_interchanges(int* rec, const int* piv_loc, int 
 // Bound: the latency of 32 dependent columns.  LU_SB columns at a time live in
 // registers (a thread owns rows tid, tid + 512, ...), so a column costs a pivot
 // reduction, one exchange of two rows through shared memory and multiply-adds;
-// the columns right of them take one rank-LU_SB update per block.  (With the
-// rank-1 updates in shared memory every column read and wrote the rest of the
-// panel: 8 MB at 2,048 rows against 1.3 MB.)  Each entry sees the same
-// operations in the same order as with rank-1 updates.
+// the columns right of them take one rank-LU_SB update per block.  Each entry
+// sees the same operations in the same order as with rank-1 updates in shared
+// memory, where every column read and wrote the rest of the panel (8 MB at 2,048
+// rows against 1.3 MB).  64 matrices, us per panel over all panels of an LU, launched
+// back to back, with rank-1 updates and now: FP32 62 and 49 at 64 rows, 78 and 57 at
+// 540, 108 and 71 at 1,152; FP64 286 and 194 at 64, 360 and 254 at 780.  The
+// unrolled columns are 35 us of instruction fetches when nothing of the kernel is
+// cached (a profiler that empties the caches, a 256 MB memset in between): FP32 64
+// and 87, 84 and 93, 113 and 106; inside a factorization the caches hold it.
 constexpr int LU_SMEM_BYTES = 200 * 1024;
 constexpr int LU_SB = 8;
 constexpr int LU_PT = 512;                       // threads of the shared-memory panel

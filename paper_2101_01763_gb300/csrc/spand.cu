@@ -42,7 +42,9 @@
 
 namespace spand {
 
-// longest operand of one apply term (bytes): larger factors are refused
+// longest operand of one apply term (bytes): larger factors are refused with
+// SPAND_ERR_UNSUPPORTED, the status that callers know; the sweeps themselves stage
+// no operand and have no such limit
 constexpr size_t kGemvTermMax = 200 * 1024;
 // dynamic shared memory of the RRQR cluster kernel (W chunk + reflector)
 constexpr size_t kQrSmemMax = 224 * 1024;   // clamped per kernel to the opt-in limit minus its static shared memory
@@ -1109,7 +1111,8 @@ static void batched_inverses(DevMem& tmp, const std::vector<MatRef<T>>& mats, co
 // of 256 x 128 p=3 took): from INV_SERIAL rows on the block recursion takes over,
 // in FP32 multiply-adds as in the kernel (that factorization and solve 837 -> 827
 // ms).  With the recursion for every size 64 x 32 p=2, of at most 268 rows, was
-// 0.2 ms slower.
+// 0.2 ms slower.  The line itself is flat (ms): 128 35.4 and 817, 320 35.1 and 819,
+// 640 35.2 and 820 for 64 x 32 p=2 and 256 x 128 p=3.
 constexpr int INV_SERIAL = 320;
 
 template <typename T>
@@ -2751,7 +2754,9 @@ static int run_phases(const Program<T>& pg, const std::vector<typename ApplyProg
                       bool capturing = false) {
   if (!capturing) note_launch(ph.size());
   for (auto& p : ph) {
-    // a phase of few tiles gets its parallelism from the warps of a tile
+    // a phase of few tiles gets its parallelism from the warps of a tile: 16 warps up to 0, 300, 600 and 1,200 tiles
+    // take 115.1, 111.9, 111.3 and 111.7 ms in a solve of 192 x 96 p=3, 84.8, 86.9, 87.1 and 87.1 in one of 75 x 33
+    // p=3 and 1.94, 1.97, 1.99 and 2.18 in an FP64 apply of 64 x 32 p=2 and its transpose
     const int threads = p.ntiles < 600 ? 32 * GV_WARPS_MAX : 256;
     auto kern = p.trans ? k_gemv<T, true, 1> : p.groups == 2 ? k_gemv<T, false, 2> : k_gemv<T, false, 1>;
     kern<<<p.ntiles, threads, 0, st>>>(p.tasks, p.terms, p.tiles, pg.partial, pg.done);
